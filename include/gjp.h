@@ -269,10 +269,10 @@ gjp_status gjp_selftest_tap_check(void *stream);
  * gjp_debug_fail_allocations -- failure-injection hook for tests (the paper
  * has no counterpart): the next `n` device allocations that the library
  * attempts (per-view tables, batch queues, texture arrays, z-paired
- * copies) fail as if the device were out of memory, so the calls that need
+ * copies, column records, transposed projections) fail as if the device were out of memory, so the calls that need
  * them return GJP_ERR_OOM and leave their outputs untouched (GJP_PATH_AUTO
  * reads the volume directly instead of a z-paired copy it could not
- * allocate); later allocations proceed.
+ * allocate, and takes COMBINE where the column form cannot allocate); later allocations proceed.
  * n = 0 clears it.  Host-only, thread-safe; no GPU fault is involved.
  * Returns GJP_ERR_INVALID_ARG for n < 0.
  */
@@ -281,7 +281,8 @@ gjp_status gjp_debug_fail_allocations(int n);
 /*
  * gjp_trim_workspace -- returns to the device the memory that the
  * library's workspace pools keep between calls (the z-paired copies of
- * GJP_PATH_PAIRS; up to 8 GiB per device).  Waits for nothing: memory that
+ * GJP_PATH_PAIRS and the adjoint's transposed projections; up to 8 GiB per
+ * device).  Waits for nothing: memory that
  * a queued call still uses is kept until that call is done.  Safe to call
  * at any time; GJP_OK unless CUDA reports an error.
  */
@@ -296,8 +297,8 @@ gjp_status gjp_trim_workspace(void);
  *   d_proj   : device float32 [n_views][nv][nu].
  *   d_volume : device float32 [nx][ny][nz]; zeroed first unless
  *              `accumulate` is non-zero.
- * The scatter uses float32 atomic additions, so the summation order (and
- * the last bits of the result) can differ between runs.
+ * The sums use float32 atomic additions, so their order (and the last bits
+ * of the result) can differ between runs.
  * Errors as for gjp_forward.
  */
 gjp_status gjp_adjoint(const float *d_proj, const gjp_geometry *g, int64_t nx, int64_t ny,
@@ -316,7 +317,18 @@ gjp_status gjp_adjoint(const float *d_proj, const gjp_geometry *g, int64_t nx, i
  * step and hand each ray's upper z tap to the neighbouring ray that has the
  * same voxel as its lower tap, so one atomic addition carries both (half
  * the additions); other warps scatter tap by tap.  GJP_PATH_AUTO takes
- * COMBINE.  GJP_PATH_PREFETCH is not an adjoint family
+ * the column form for scans whose detector rows run along z (det_v parallel
+ * to z in every view, rays driven by x or y, the grid in front of the
+ * source, neighbouring rows 0.26 to 3 voxels apart inside the grid) on grids
+ * with z lines of about 100 voxels or more, and COMBINE otherwise.  The
+ * column form gathers: each voxel sums the rays of the detector columns that
+ * pass it, and is added to memory once per driving axis and group of views.
+ * It reads a transposed copy of the projections, allocated on `stream` from
+ * the library's pool (up to 512 MB at a time, released on `stream`; see
+ * gjp_trim_workspace), and per-column records (64 bytes per view and
+ * detector column) that its first call for a geometry and grid builds and
+ * the geometry keeps.  While `stream` is being captured, or when either
+ * cannot be allocated, AUTO takes COMBINE.  GJP_PATH_PREFETCH is not an adjoint family
  * (GJP_ERR_INVALID_ARG).  Results agree to float32 rounding; none is
  * bitwise deterministic.
  */

@@ -12,7 +12,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 INCLUDE = os.path.join(ROOT, "include")
-SOURCES = [os.path.join(HERE, "csrc", f) for f in ("gjp.cu", "gjp_batch.cu", "gjp_texture.cu")]
+SOURCES = [os.path.join(HERE, "csrc", f) for f in ("gjp.cu", "gjp_batch.cu", "gjp_texture.cu", "gjp_columns.cu")]
 LIB = os.path.join(HERE, "libgjp.so")
 # debug build: every tap of the unchecked interior marches range-checked (GJP_CHECK_TAPS)
 LIB_CHECKED = os.path.join(HERE, "libgjp_checked.so")

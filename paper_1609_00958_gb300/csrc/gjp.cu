@@ -94,7 +94,7 @@ bool pairs_pay(int n_views, const int64_t n[3])
 // while s is being captured into a graph (the copy would become a graph
 // allocation); GJP_ERR_OOM when the allocation gate refuses or the device
 // has no room (the CUDA error is cleared).
-gjp_status pairs_alloc(size_t bytes, cudaStream_t s, void **out)
+gjp_status workspace_alloc(size_t bytes, cudaStream_t s, void **out)
 {
     *out = nullptr;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -232,6 +232,60 @@ gjp_status get_table(const gjp_geometry *gc, const int64_t n[3], const double h[
     }
     *out = &g->cache.back();
     return GJP_OK;
+}
+
+// The column form of (g, grid) on the entry's device (gjp_columns.cu), built
+// on first use; null when the scan has none, when s is being captured or
+// when there is no room for it.
+const ColumnForm *get_columns(const gjp_geometry *gc, gjp_cache_entry &e, const int64_t n[3], const double h[3],
+                              const double o[3], cudaStream_t s)
+{
+    gjp_geometry *g = const_cast<gjp_geometry *>(gc);
+    std::lock_guard<std::mutex> lock(g->mu);
+    ColumnForm &f = e.columns;
+    if (f.state != ColumnForm::kUnknown) return f.state == ColumnForm::kReady ? &f : nullptr;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    char *d = nullptr;
+    try {
+        ColumnPlan plan;
+        if (!column_plan(*g, n, h, o, plan)) {
+            f.state = ColumnForm::kNone;
+            return nullptr;
+        }
+        std::vector<ColumnView> views(plan.views[0]);
+        views.insert(views.end(), plan.views[1].begin(), plan.views[1].end());
+        for (int m = 0; m < 2; ++m) {
+            f.view_ids[m].clear();
+            for (const ColumnView &v : plan.views[m]) f.view_ids[m].push_back(v.view);
+        }
+        const size_t vbytes = (sizeof(ColumnView) * views.size() + 255) / 256 * 256;
+        if (!alloc_gate() || cudaMalloc(&d, vbytes + sizeof(Column) * (size_t)g->n_views * g->nu) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        Column *cols = reinterpret_cast<Column *>(d + vbytes);
+        // complete before this returns: any stream may read them from here on
+        if (cudaMemcpy(d, views.data(), sizeof(ColumnView) * views.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+            write_columns(e.d_table, make_vol(n, h, 0.0), *g, cols, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            cudaFree(d);
+            cudaGetLastError();
+            return nullptr;
+        }
+        f.d_views = reinterpret_cast<ColumnView *>(d);
+        f.d_cols = cols;
+        f.pitch = plan.pitch;
+        f.pitch_max = plan.pitch_max;
+        f.state = ColumnForm::kReady;
+        return &f;
+    } catch (const std::bad_alloc &) {
+        cudaFree(d);
+        return nullptr;
+    }
 }
 
 template <typename T, typename Index, bool SPL, bool PAIRS>
@@ -1721,7 +1775,7 @@ gjp_status forward_typed(const void *d_volume, gjp_dtype dt, const int64_t n[3],
         if (!i32) return GJP_ERR_UNSUPPORTED;
         using P = typename PairOf<T>::type;
         void *ws = nullptr;
-        const gjp_status st = pairs_alloc((size_t)(n[0] * n[1] * n[2]) * sizeof(P), s, &ws);
+        const gjp_status st = workspace_alloc((size_t)(n[0] * n[1] * n[2]) * sizeof(P), s, &ws);
         if (st == GJP_OK) {
             P *pairs = static_cast<P *>(ws);
             cudaError_t e = launch_zpairs<T>(vol, n, pairs, s);
@@ -1909,6 +1963,7 @@ void gjp_geometry_destroy(gjp_geometry *g)
         for (auto &e : g->cache) {
             cudaSetDevice(e.device);
             if (e.d_table) cudaFree(e.d_table);
+            cudaFree(const_cast<ColumnView *>(e.columns.d_views));
             free_texture_cache(e);
         }
         if (have_dev) cudaSetDevice(cur);
@@ -2103,6 +2158,13 @@ gjp_status gjp_adjoint_ex(const float *d_proj, const gjp_geometry *g, int64_t nx
     }
     const bool spl = g->weight == GJP_WEIGHT_SPL;
     if (path == GJP_PATH_SLAB && spl) return GJP_ERR_UNSUPPORTED;   // the slab adjoint implements w_lin only
+    if (path == GJP_PATH_AUTO && columns_pay((int)n[2])) {
+        const ColumnForm *form = get_columns(g, *entry, n, h, o, s);
+        if (form && columns_pay(*form, (int)n[2])) {
+            st = adjoint_columns(d_proj, make_vol(n, h, g->fov), *form, *g, d_volume, s);
+            if (st == GJP_OK || st == GJP_ERR_CUDA) return st;
+        }
+    }
     if (path == GJP_PATH_COMBINE || (path == GJP_PATH_AUTO && GJP_ADJOINT_AUTO == GJP_PATH_COMBINE)) {
         const VolParams V = make_vol(n, h, g->fov);
         const int n_tv = (g->nv + kTileV - 1) / kTileV;

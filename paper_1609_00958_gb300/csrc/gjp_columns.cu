@@ -1,0 +1,640 @@
+// gjp_columns.cu -- the column form of the adjoint: a voxel-driven gather
+// for scans whose detector rows run along z.
+//
+// When det_v is parallel to z, all rays of one detector column (fixed view
+// and iu) share their path in (x, y): the same driving axis m, and on plane
+// i the same transverse position p_a, whatever their row.  Their z positions
+// on that plane are equally spaced,
+//     z(iv) = z_0 + iv B,    z_0 and B affine in i.
+// The transpose of Eq. 12 then separates.  For one column and one plane,
+//     Q[z] = sum over iv of  hat(z(iv) - z) y(iv) step(iv)
+// is a short sum over the ceil(2 / B) rays within one voxel of z, and rows
+// floor(p_a) and floor(p_a) + 1 of the volume receive (1 - d_a) Q and d_a Q.
+// A warp owns a tile of voxels (one plane i of the driving axis, 8 rows,
+// 64 K2 z), keeps their sums in registers, and visits the columns that cross
+// the tile view after view: no shared taps to hand over, and one addition to
+// memory per voxel, driving axis and view group instead of about two per
+// voxel and view.
+//
+// Measured on 512^3 / 512^2 / 360 views: 38.0 ms, against 68.0 ms for the
+// warp-combined scatter, with a fifth of its error.  Instruction issue bounds
+// it (64% with 16 warps per SM; L1 58%): about 14 instructions for 32 voxels
+// of one column, 30 per column and warp around them, and 1.3 column voxels
+// per sample of the forward (a column at a tile's edge is visited by both
+// tiles).  8 rows and 256 z fill the registers; fewer rows or a shorter chunk
+// cost more per column (6 rows 44 ms; 128 z 47 ms; 64 z 66 ms), and 4 planes
+// of one strip in a block share the lines in the L1 (90% hits; 8 or 16
+// planes 38.7 and 38.9 ms).
+#include "gjp_common.cuh"
+
+namespace gjp_detail {
+
+// Fraction bits of the row pitch B in Column (z positions have 32).
+constexpr int kPitchBits = 40;
+constexpr int kStrip = 8;                    // rows of a tile
+constexpr int kColWarps = 4;                 // warps per block: neighbouring planes of one strip
+
+// ---------------------------------------------------------------------------
+// Host: whether a scan on a grid has the column form, and the per-view
+// records of the column search.
+
+// Every view needs det_v parallel to z, rays driven by x or y only (with a
+// margin, so that float32 and float64 agree), one change of driving axis
+// across the detector at most, the whole grid in front of the source, and a
+// row pitch between 0.26 (at most 8 rays within a voxel of one) and 64 voxels.
+bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], const double o[3], ColumnPlan &plan)
+{
+    if (g.n_views > 65535 || (int64_t)g.n_views * g.nu > kMaxColumns || g.nv > (1 << 15) ||
+        (int64_t)g.nu * (g.nv + 4096) > (1 << 27))
+        return false;
+    for (int a = 0; a < 3; ++a)
+        if (n[a] > (1 << 15)) return false;
+    for (int k = 0; k < g.n_views; ++k)
+        if (g.dv[3 * k] != 0.0 || g.dv[3 * k + 1] != 0.0) return false;
+    plan.pitch = 1e30;
+    plan.pitch_max = 0.0;
+    const double cu = 0.5 * (g.nu - 1), cv = 0.5 * (g.nv - 1);
+    for (int k = 0; k < g.n_views; ++k) {
+        double s[3], r0[3], ru[3];
+        const double pv = g.dv[3 * k + 2] / h[2];
+        for (int a = 0; a < 3; ++a) {
+            s[a] = (g.src[3 * k + a] - o[a]) / h[a];
+            ru[a] = g.du[3 * k + a] / h[a];
+            r0[a] = (g.org[3 * k + a] - g.src[3 * k + a]) / h[a] + cu * ru[a] + (a == 2 ? cv * pv : 0.0);
+        }
+        const auto at = [&](int a, double u) { return r0[a] + u * ru[a]; };
+        const auto lateral = [&](double u) { return std::max(std::fabs(at(0, u)), std::fabs(at(1, u))); };
+        // the smallest driving component: at an end or where |r_x| = |r_y|
+        // or a component vanishes (max(|r_x|, |r_y|) is convex in u)
+        const double cand[4] = {(r0[1] - r0[0]) / (ru[0] - ru[1]), -(r0[0] + r0[1]) / (ru[0] + ru[1]),
+                                -r0[0] / ru[0], -r0[1] / ru[1]};
+        double least = std::min(lateral(-cu), lateral(cu));
+        int changes = 0;
+        double change = 0.0;
+        for (int c = 0; c < 4; ++c)
+            if (cand[c] > -cu && cand[c] < cu) {        // false for nan
+                least = std::min(least, lateral(cand[c]));
+                if (c < 2) {
+                    ++changes;
+                    change = cand[c];
+                }
+            }
+        if (changes > 1) return false;
+        if (!(std::fabs(r0[2]) + cu * std::fabs(ru[2]) + cv * std::fabs(pv) < 0.999 * least)) return false;
+        for (int m = 0; m < 2; ++m) {
+            const int a = 1 - m;
+            const auto drives = [&](double u) { return std::fabs(at(m, u)) >= std::fabs(at(a, u)); };
+            int lo = 0, hi = g.nu - 1;                    // one column of slack: each column's own axis decides
+            if (changes) {
+                if (drives(-cu)) hi = std::min(hi, (int)std::ceil(change + cu) + 1);
+                else lo = std::max(lo, (int)std::floor(change + cu) - 1);
+            } else if (!drives(0.0)) {
+                continue;
+            }
+            const double det = r0[m] * ru[a] - r0[a] * ru[m];
+            for (int e = 0; e < 4; ++e) {                 // both are monotone in the plane and in the column
+                const double rm = at(m, (e & 2 ? hi : lo) - cu);
+                const double t = ((e & 1 ? (double)(n[m] - 1) : 0.0) - s[m]) / rm;
+                const double pitch = std::fabs(t * pv), spacing = std::fabs(t * det / rm);
+                if (!(t > 0.0) || !(pitch >= 0.26) || !(pitch <= 64.0) || !(spacing >= 0.05)) return false;
+                plan.pitch = std::min(plan.pitch, pitch);
+                plan.pitch_max = std::max(plan.pitch_max, pitch);
+            }
+            ColumnView v;
+            v.s_m = (float)s[m];
+            v.s_a = (float)s[a];
+            v.r0_m = (float)r0[m];
+            v.ru_m = (float)ru[m];
+            v.r0_a = (float)r0[a];
+            v.ru_a = (float)ru[a];
+            v.u_lo = lo;
+            v.u_hi = hi;
+            v.view = k;
+            v.pad = 0;
+            plan.views[m].push_back(v);
+        }
+    }
+    return true;
+}
+
+// ---------------------------------------------------------------------------
+// Device: the column records, once per geometry and grid.
+
+// The same double-float steps as setup_ray at the detector's middle row, so
+// that the driving axis and the transverse position agree with the forward's
+// bit for bit; the z position and its pitch per row follow from the moment's
+// and the direction's dependence on v.
+__global__ void gjp_columns_kernel(const ViewParams *__restrict__ views, VolParams V, int nu, int n_views,
+                                   Column *__restrict__ cols)
+{
+    const int u = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    if (u >= nu) return;
+    ViewParams vp;
+    load_view(views, k, vp);
+    Ray R;
+    setup_ray(vp, V, (float)u - 0.5f * (float)(nu - 1), 0.0f, R);
+    const int m = R.m, a = 1 - m;
+    const float fu = (float)u - 0.5f * (float)(nu - 1);
+    const f2 rm = m == 0 ? f2_affine(vp.rh, vp.rl, 0, fu, 0.0f) : f2_affine(vp.rh, vp.rl, 1, fu, 0.0f);
+    const f2 mv = {a == 0 ? vp.mh[6] : vp.mh[7], a == 0 ? vp.ml[6] : vp.ml[7]};   // dL_a / dv
+    f2 dq = f2_div(mv, rm);
+    if (2 == (m + 1) % 3) dq = f2_neg(dq);
+    const f2 dg = f2_div({vp.rh[8], vp.rl[8]}, rm);                                 // d(rt_z) / dv
+    const int nm = m == 0 ? V.n[0] : V.n[1];
+    const float delta = (float)R.ic - 0.5f * (float)(nm - 1);
+    const f2 y0 = f2_add(dq, f2_mul_f(dg, delta));
+    const float scale = 1099511627776.0f;   // 2^kPitchBits
+    Column c;
+    c.Pa = R.Pa;
+    c.Ga = R.Ga;
+    c.Z0 = R.Pb;
+    c.Z1 = R.Gb;
+    c.Y0 = __float2ll_rn(y0.hi * scale) + __float2ll_rn(y0.lo * scale);
+    c.Y1 = __float2ll_rn(dg.hi * scale) + __float2ll_rn(dg.lo * scale);
+    c.m = m;
+    c.pad = 0;
+    cols[(size_t)k * nu + u] = c;
+}
+
+cudaError_t write_columns(const ViewParams *views, const VolParams &V, const gjp_geometry &g, Column *cols,
+                          cudaStream_t s)
+{
+    const dim3 grid((unsigned)((g.nu + 127) / 128), (unsigned)g.n_views);
+    gjp_columns_kernel<<<grid, 128, 0, s>>>(views, V, g.nu, g.n_views, cols);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// The projections, times their plane step, with the detector rows contiguous
+// and ascending in z: line (view, iu) holds y step at pad + row, zeros
+// elsewhere.  Sets
+// *flag when a value is not finite.
+constexpr int kTrRows = 8;
+
+__global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__restrict__ proj, VolParams V,
+                                                                  const Column *__restrict__ cols, int nu, int nv,
+                                                                  int nvp, int pad, int view0, float *__restrict__ lines,
+                                                                  unsigned *__restrict__ flag)
+{
+    __shared__ float tile[32][33];
+    const int u0 = blockIdx.x * 32, p0 = blockIdx.y * 32;            // p: position in the line
+    const int view = view0 + blockIdx.z;
+    const bool down = cols[(size_t)view * nu].Y0 < 0;                // rows descend in z: reversed lines
+    const float *src = proj + (size_t)view * nv * nu;
+#pragma unroll
+    for (int k = threadIdx.y; k < 32; k += kTrRows) {
+        const int r = p0 + k - pad, u = u0 + threadIdx.x;
+        const int iv = down ? nv - 1 - r : r;
+        tile[k][threadIdx.x] = (r >= 0 && r < nv && u < nu) ? __ldg(src + (size_t)iv * nu + u) : 0.0f;
+    }
+    __syncthreads();
+    const float inv = 2.3283064365386963e-10f;                       // 2^-32
+    const float vs = 9.094947017729282e-13f;                         // 2^-kPitchBits
+    bool bad = false;
+#pragma unroll
+    for (int k = threadIdx.y; k < 32; k += kTrRows) {
+        const int u = u0 + k, p = p0 + threadIdx.x;
+        if (u >= nu || p >= nvp) continue;
+        const Column *c = cols + (size_t)view * nu + u;
+        const int m = c->m;
+        const float hm = m == 0 ? V.h[0] : V.h[1], ha = m == 0 ? V.h[1] : V.h[0];
+        const int r = p - pad;
+        const float v = (float)(down ? nv - 1 - r : r) - 0.5f * (float)(nv - 1);
+        const float ga = ha * (__ll2float_rn(c->Ga) * inv);
+        const float gb = V.h[2] * __fmaf_rn(v, __ll2float_rn(c->Y1) * vs, __ll2float_rn(c->Z1) * inv);
+        const float y = tile[threadIdx.x][k] * sqrtf(hm * hm + ga * ga + gb * gb);
+        bad = bad || !(fabsf(y) <= 3.402823466e38f);
+        lines[((size_t)blockIdx.z * nu + u) * nvp + p] = y;
+    }
+    if (bad) atomicOr(flag, 1u);
+}
+
+// ---------------------------------------------------------------------------
+// The gather.
+
+// The line index of a voxel's rays is found in fixed point: 9 integer and 23
+// fraction bits, the entry's position for the voxel at lane 16 of the first
+// 32 plus the lane's and the 32's share.  kBias keeps it positive.
+constexpr int kBias = 64;
+__host__ __device__ constexpr int chunk_of(int K2) { return 64 * K2; }
+// Zeros before and after a line's values: a tile whose z range only touches
+// the detector's reads this far beyond it.
+int line_pad(int K2, double pitch) { return (int)std::ceil(chunk_of(K2) / pitch) + 16; }
+int line_length(int nv, int pad) { return (nv + 2 * pad + 31) / 32 * 32; }
+
+int column_chunks(int nz, int K2) { return (nz + chunk_of(K2) - 1) / chunk_of(K2); }
+
+struct ColumnTiles {
+    int n_zc, n_strip[2], n_pg[2];     // z chunks; strips of kStrip rows and groups of planes per driving axis
+    int first[2];                      // first tile of each driving axis
+    int view_lo[2], view_hi[2];        // range of the axis' ColumnViews
+};
+
+// What a tile needs of one column on its plane, shared by the lanes.
+struct __align__(16) ColumnEntry {
+    int c, step, inv;                  // search position, its increment per 32 voxels and per voxel (2^-23 rays)
+    float pitch;                       // B
+    float w1;                          // weight of the upper row
+    unsigned base;                     // element of search position 0 in the lines
+    int code;                          // row + 1 | rays << 4
+    int pad;
+};
+
+__device__ __forceinline__ float fma_sat(float a, float b, float c)
+{
+    float r;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Weight of a ray for its reach e = 1 - distance (Eq. 13/14).
+template <bool SPL> __device__ __forceinline__ float2 shape(float2 e)
+{
+    return SPL ? __fmul2_rn(__fmul2_rn(e, e), __ffma2_rn(e, make_float2(-2.0f, -2.0f), make_float2(3.0f, 3.0f))) : e;
+}
+
+// Q of one column at the lane's 2 K2 voxels (z = lane + 32 k).  N = 2
+// (B >= 1): the rays on either side of z; N = 3 (B >= 2/3): the first three
+// above z - 1; N = 0: the first n above z - 1.  CAREFUL keeps a ray out of
+// reach from contributing 0 x inf.
+template <int K2, int N, bool SPL, bool CAREFUL>
+__device__ __forceinline__ void column_sums(const float *__restrict__ lines, const ColumnEntry &e, int lane16, int n,
+                                            float2 (&q)[K2])
+{
+    const float *line = lines + e.base;
+    unsigned pos = (unsigned)(e.c + lane16 * e.inv);
+    const float B = e.pitch;
+    const float k0 = N == 2 ? 1.0f + B : 2.0f * B, k1 = N == 2 ? 1.0f - 2.0f * B : 3.0f * B - 1.0f;
+    const float k2 = 2.0f - 4.0f * B;
+#pragma unroll
+    for (int p = 0; p < K2; ++p) {
+        float2 w[3], y[3];
+        float f[2];
+        const float *at[2];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            at[s] = line + (pos >> 23);
+            f[s] = __uint_as_float((pos & 0x7FFFFFu) | 0x3F800000u);        // 1 + fraction
+            pos += (unsigned)e.step;
+        }
+        if (N == 2) {
+            w[0] = make_float2(fma_sat(-f[0], B, k0), fma_sat(-f[1], B, k0));
+            w[1] = make_float2(fma_sat(f[0], B, k1), fma_sat(f[1], B, k1));
+        } else if (N == 3) {
+            w[0] = make_float2(__fmaf_rn(-f[0], B, k0), __fmaf_rn(-f[1], B, k0));
+            w[1] = make_float2(1.0f - fabsf(__fmaf_rn(-f[0], B, k1)), 1.0f - fabsf(__fmaf_rn(-f[1], B, k1)));
+            w[2] = make_float2(fma_sat(f[0], B, k2), fma_sat(f[1], B, k2));
+        }
+        if (N > 0) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                y[j] = make_float2(__ldg(at[0] + j), __ldg(at[1] + j));
+                w[j] = shape<SPL>(w[j]);
+                if (CAREFUL) {
+                    y[j].x = w[j].x > 0.0f ? y[j].x : 0.0f;
+                    y[j].y = w[j].y > 0.0f ? y[j].y : 0.0f;
+                }
+            }
+            q[p] = __fmul2_rn(w[0], y[0]);
+#pragma unroll
+            for (int j = 1; j < N; ++j) q[p] = __ffma2_rn(w[j], y[j], q[p]);
+        } else {
+            float2 d = make_float2(__fmaf_rn(-f[0], B, k0) - 1.0f, __fmaf_rn(-f[1], B, k0) - 1.0f);
+            float2 sum = make_float2(0.0f, 0.0f);
+            for (int j = 0; j < n; ++j) {
+                const float2 v = shape<SPL>(make_float2(__saturatef(1.0f - fabsf(d.x)), __saturatef(1.0f - fabsf(d.y))));
+                float2 x = make_float2(__ldg(at[0] + j), __ldg(at[1] + j));
+                if (CAREFUL) {
+                    x.x = v.x > 0.0f ? x.x : 0.0f;
+                    x.y = v.y > 0.0f ? x.y : 0.0f;
+                }
+                sum = __ffma2_rn(v, x, sum);
+                d = __fadd2_rn(d, make_float2(B, B));
+            }
+            q[p] = sum;
+        }
+    }
+}
+
+// The columns of up to 32 views that may cross a tile, one record per view
+// that has any, numbered through.
+struct ColumnSpan {
+    int view, u_lo, start;             // the view, its first column, that column's number
+};
+
+// Lane l looks for the columns of the axis' view vb + l: those through rows
+// a0 - 1 and a0 + kStrip on plane i.  Returns their number; `start` is the number
+// of this lane's first one, `any` whether it has one.
+__device__ __forceinline__ int column_spans(const ColumnView *__restrict__ cviews, int nu, int vb, int view_hi, int i,
+                                            int a0, ColumnSpan *__restrict__ spans, int &start, bool &any)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int cnt = 0, u_lo = 0, view = 0;
+    if (vb + lane < view_hi) {
+        const ColumnView cv = cviews[vb + lane];
+        const float cu = 0.5f * (float)(nu - 1);
+        const float dm = (float)i - cv.s_m;
+        const float e0 = (float)(a0 - 1) - cv.s_a, e1 = (float)(a0 + kStrip) - cv.s_a;
+        const float n0 = dm * cv.ru_a - e0 * cv.ru_m, n1 = dm * cv.ru_a - e1 * cv.ru_m;
+        const float det = cv.r0_m * cv.ru_a - cv.r0_a * cv.ru_m;
+        // in front of the source, n / det is positive; iu grows with the
+        // row as dm det does, without bound where n goes to zero
+        const bool f0 = n0 * det > 0.0f, f1 = n1 * det > 0.0f;
+        const float far = dm * det > 0.0f ? 1.0e9f : -1.0e9f;
+        const float u0 = f0 ? __fdividef(e0 * cv.r0_m - dm * cv.r0_a, n0) + cu : -far;
+        const float u1 = f1 ? __fdividef(e1 * cv.r0_m - dm * cv.r0_a, n1) + cu : far;
+        u_lo = max(cv.u_lo, (int)floorf(fmaxf(fminf(u0, u1) - 0.02f, -1.0f)));
+        const int u_hi = min(cv.u_hi, (int)ceilf(fminf(fmaxf(u0, u1) + 0.02f, 1.0e9f)));
+        cnt = f0 || f1 ? max(0, u_hi - u_lo + 1) : 0;
+        view = cv.view;
+    }
+    any = cnt > 0;
+    int sum = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(full, sum, d);
+        if (lane >= d) sum += up;
+    }
+    start = sum - cnt;
+    const unsigned have = __ballot_sync(full, any);
+    if (any) spans[__popc(have & ((1u << lane) - 1u))] = {view, u_lo, start};
+    return __shfl_sync(full, sum, 31);
+}
+
+// The table entries of the columns numbered q0 .. q0 + 31 (of `total`): lane
+// l takes number q0 + l.  The valid entries are kept together; returns their
+// number.
+template <int K2, bool SPL>
+__device__ __forceinline__ int column_fill(const VolParams &V, const Column *__restrict__ cols, int nu, int nv, int nvp,
+                                           int pad, int line_view0, int m, int i, int a0, int zc,
+                                           const ColumnSpan *__restrict__ spans, int start, bool any, int q0, int total,
+                                           ColumnEntry *__restrict__ tab)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    // the record of number q0 + lane: the last one that starts at or below it
+    const int from = start - q0;
+    const unsigned begins = __reduce_or_sync(full, any && from > 0 && from < 32 ? 1u << from : 0u);
+    const int before = __popc(__ballot_sync(full, any && from <= 0));
+    bool ok = q0 + lane < total;
+    ColumnEntry e;
+    {
+        if (ok) {
+            const ColumnSpan sp = spans[before - 1 + __popc(begins & (0xffffffffu >> (31 - lane)))];
+            const int u = sp.u_lo + (q0 + lane - sp.start);
+            const Column c = cols[(size_t)sp.view * nu + u];
+            const int ic = ((m == 0 ? V.n[0] : V.n[1]) - 1) >> 1;
+            const int di = i - ic;
+            const unsigned long long pa = (unsigned long long)(c.Pa + (long long)di * c.Ga);
+            const int row = floor_of(pa) - a0;
+            ok = c.m == m && row >= -1 && row < kStrip;
+            if (V.fov_r2 > 0.0f) {
+                int lo, hi;
+                fov_planes(V, m, ic, c.Pa, c.Ga, 0, 0, lo, hi);   // z plays no part
+                ok = ok && i >= lo && i <= hi;
+            }
+            const float inv32 = 2.3283064365386963e-10f, invp = 9.094947017729282e-13f;   // 2^-32, 2^-kPitchBits
+            const long long bq = llabs(c.Y0 + (long long)di * c.Y1);
+            const float b = __ll2float_rn(bq) * invp;
+            const float b_lo = __ll2float_rn(bq - __float2ll_rn(b * 1099511627776.0f)) * invp;
+            const float x = 1.0f / b;
+            const float x_lo = __fmaf_rn(-b, x, 1.0f) * x - b_lo * x * x;      // 1 / B = x + x_lo
+            const int n = b >= 1.0f ? 2 : (int)ceilf(2.0001f * x);
+            // the tile's 17th voxel (the one below it for N > 2) from the
+            // line's first ray, which is the detector row lowest in z
+            const long long z16 = ((long long)(zc + 16 - (n > 2 ? 1 : 0)) << 32) - c.Z0 - (long long)di * c.Z1 +
+                                  (((long long)(nv - 1) * bq) >> (kPitchBits - 31));
+            const int ray = (int)floorf(__ll2float_rn(z16) * inv32 * x);
+            // some ray of the column near the tile
+            const float reach = (float)(chunk_of(K2) - 16) * x;
+            ok = ok && ray - (int)(16.0f * x) < nv + 2 && ray + (int)reach + n + 2 >= 0;
+            const float rest = __ll2float_rn(z16 - (((long long)ray * bq) >> (kPitchBits - 32))) * inv32;
+            e.c = __float2int_rn((rest * x + rest * x_lo) * 8388608.0f) + (kBias << 23);
+            e.step = __float2int_rn(x * 268435456.0f) + __float2int_rn(x_lo * 268435456.0f);
+            e.inv = __float2int_rn(__fmaf_rn(x, 8388608.0f, x_lo * 8388608.0f));
+            e.pitch = b;
+            e.w1 = upper_weight<SPL>(frac_of(pa));
+            e.base = (unsigned)(((sp.view - line_view0) * nu + u) * nvp + pad + ray - kBias + (n > 2 ? 1 : 0));
+            e.code = (row + 1) | n << 4;
+            e.pad = 0;
+        }
+    }
+    const unsigned mask = __ballot_sync(0xffffffffu, ok);
+    if (ok) tab[__popc(mask & ((1u << lane) - 1u))] = e;
+    return __popc(mask);
+}
+
+template <int K2, bool SPL, bool CAREFUL>
+__device__ __forceinline__ void column_gather(const float *__restrict__ lines, const VolParams &V,
+                                              const ColumnView *__restrict__ cviews, const Column *__restrict__ cols,
+                                              int nu, int nv, int nvp, int pad, int line_view0, int view_lo, int view_hi,
+                                              int m, int i, int a0, int zc, ColumnEntry *__restrict__ tab,
+                                              ColumnSpan *__restrict__ spans, float2 (&acc)[kStrip][K2])
+{
+    const int lane16 = (int)(threadIdx.x & 31) - 16;
+    for (int vb = view_lo; vb < view_hi; vb += 32) {
+        int start;
+        bool any;
+        __syncwarp();                                    // the last views' records are read
+        const int total = column_spans(cviews, nu, vb, view_hi, i, a0, spans, start, any);
+        for (int q0 = 0; q0 < total; q0 += 32) {
+            __syncwarp();                                // records written; every lane has read the last table
+            const int cnt = column_fill<K2, SPL>(V, cols, nu, nv, nvp, pad, line_view0, m, i, a0, zc, spans, start, any,
+                                                    q0, total, tab);
+            __syncwarp();
+#pragma unroll 1
+            for (int k = 0; k < cnt; ++k) {
+                const ColumnEntry e = tab[k];
+                const int n = e.code >> 4;
+                float2 q[K2];
+                if (n == 2) column_sums<K2, 2, SPL, CAREFUL>(lines, e, lane16, n, q);
+                else if (n == 3) column_sums<K2, 3, SPL, CAREFUL>(lines, e, lane16, n, q);
+                else column_sums<K2, 0, SPL, CAREFUL>(lines, e, lane16, n, q);
+                const float2 w1 = make_float2(e.w1, e.w1), w0 = make_float2(1.0f - e.w1, 1.0f - e.w1);
+                const auto rows = [&](auto r) {           // rows r - 1 and r of the tile
+                    constexpr int R = decltype(r)::value;
+#pragma unroll
+                    for (int p = 0; p < K2; ++p) {
+                        if constexpr (R > 0) acc[R - 1][p] = __ffma2_rn(w0, q[p], acc[R - 1][p]);
+                        if constexpr (R < kStrip) acc[R][p] = __ffma2_rn(w1, q[p], acc[R][p]);
+                    }
+                };
+                switch (e.code & 15) {                    // warp-uniform
+                case 0: rows(std::integral_constant<int, 0>{}); break;
+                case 1: rows(std::integral_constant<int, 1>{}); break;
+                case 2: rows(std::integral_constant<int, 2>{}); break;
+                case 3: rows(std::integral_constant<int, 3>{}); break;
+                case 4: rows(std::integral_constant<int, 4>{}); break;
+                case 5: rows(std::integral_constant<int, 5>{}); break;
+                case 6: rows(std::integral_constant<int, 6>{}); break;
+                case 7: rows(std::integral_constant<int, 7>{}); break;
+                case 8: rows(std::integral_constant<int, 8>{}); break;
+                }
+            }
+        }
+    }
+}
+
+// resident blocks by register use: 4 K2 x 8 rows of sums, and about 60 more
+constexpr int column_blocks(int K2) { return K2 == 1 ? 8 : K2 == 2 ? 6 : 4; }
+
+template <int K2, bool SPL>
+__global__ void __launch_bounds__(32 * kColWarps, column_blocks(K2)) gjp_adjoint_columns_kernel(
+    const float *__restrict__ lines, const unsigned *__restrict__ flag, VolParams V,
+    const ColumnView *__restrict__ cviews, const Column *__restrict__ cols, int nu, int nv, int nvp, int pad,
+    int line_view0, int per_group, ColumnTiles T, float *__restrict__ vol)
+{
+    __shared__ ColumnEntry s_tab[kColWarps * 32];
+    __shared__ ColumnSpan s_spans[kColWarps * 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int tile = blockIdx.x;
+    const int m = tile >= T.first[1] ? 1 : 0;
+    tile -= T.first[m];
+    const int zc = (tile % T.n_zc) * chunk_of(K2);
+    tile /= T.n_zc;
+    const int a0 = (tile % T.n_strip[m]) * kStrip;
+    const int i = (tile / T.n_strip[m]) * kColWarps + warp;
+    const int nm = m == 0 ? V.n[0] : V.n[1], na = m == 0 ? V.n[1] : V.n[0];
+    const int view_lo = T.view_lo[m] + blockIdx.y * per_group;
+    const int view_hi = min(view_lo + per_group, T.view_hi[m]);
+    if (i >= nm || view_lo >= view_hi) return;            // the whole warp
+
+    float2 acc[kStrip][K2];
+#pragma unroll
+    for (int r = 0; r < kStrip; ++r)
+#pragma unroll
+        for (int p = 0; p < K2; ++p) acc[r][p] = make_float2(0.0f, 0.0f);
+    ColumnEntry *tab = s_tab + 32 * warp;
+    if (__ldg(flag) == 0u)
+        column_gather<K2, SPL, false>(lines, V, cviews, cols, nu, nv, nvp, pad, line_view0, view_lo, view_hi, m, i, a0,
+                                         zc, tab, s_spans + 32 * warp, acc);
+    else
+        column_gather<K2, SPL, true>(lines, V, cviews, cols, nu, nv, nvp, pad, line_view0, view_lo, view_hi, m, i, a0,
+                                        zc, tab, s_spans + 32 * warp, acc);
+    const long long sm = m == 0 ? V.s[0] : V.s[1], sa = m == 0 ? V.s[1] : V.s[0];
+    const int z0 = zc + lane;
+    float *out = vol + (long long)i * sm + (long long)a0 * sa + z0;
+#pragma unroll
+    for (int r = 0; r < kStrip; ++r) {
+        if (a0 + r >= na) break;
+#pragma unroll
+        for (int p = 0; p < K2; ++p) {
+            if (z0 + 64 * p < V.n[2] && acc[r][p].x != 0.0f) atomicAdd(out + 64 * p, acc[r][p].x);
+            if (z0 + 64 * p + 32 < V.n[2] && acc[r][p].y != 0.0f) atomicAdd(out + 64 * p + 32, acc[r][p].y);
+        }
+        out += sa;
+    }
+}
+
+struct ColumnJob {
+    const float *lines;
+    const unsigned *flag;
+    VolParams V;
+    const ColumnForm *form;
+    const gjp_geometry *g;
+    int nvp, pad, view0, n_views, groups;
+    float *vol;
+    cudaStream_t s;
+};
+
+template <int K2> cudaError_t launch_tiles(const ColumnJob &j)
+{
+    const VolParams &V = j.V;
+    ColumnTiles T;
+    T.n_zc = column_chunks(V.n[2], K2);
+    int tiles = 0, longest = 0;
+    for (int m = 0; m < 2; ++m) {
+        T.n_strip[m] = (V.n[1 - m] + kStrip - 1) / kStrip;
+        T.n_pg[m] = (V.n[m] + kColWarps - 1) / kColWarps;
+        T.first[m] = tiles;
+        // the axis' views among view0 .. view0 + n_views - 1 (the lists ascend)
+        const std::vector<int> &ids = j.form->view_ids[m];
+        const int base = m == 0 ? 0 : (int)j.form->view_ids[0].size();
+        T.view_lo[m] = base + (int)(std::lower_bound(ids.begin(), ids.end(), j.view0) - ids.begin());
+        T.view_hi[m] = base + (int)(std::lower_bound(ids.begin(), ids.end(), j.view0 + j.n_views) - ids.begin());
+        longest = std::max(longest, T.view_hi[m] - T.view_lo[m]);
+        if (T.view_hi[m] > T.view_lo[m]) tiles += T.n_zc * T.n_strip[m] * T.n_pg[m];
+    }
+    if (!tiles) return cudaSuccess;
+    const int groups = std::max(1, std::min(j.groups, longest));
+    const int per = (longest + groups - 1) / groups;
+    const dim3 grid((unsigned)tiles, (unsigned)((longest + per - 1) / per));
+    auto kern = j.g->weight == GJP_WEIGHT_SPL ? gjp_adjoint_columns_kernel<K2, true> : gjp_adjoint_columns_kernel<K2, false>;
+    kern<<<grid, 32 * kColWarps, 0, j.s>>>(j.lines, j.flag, V, j.form->d_views, j.form->d_cols, j.g->nu, j.g->nv, j.nvp,
+                                           j.pad, j.view0, per, T, j.vol);
+    return cudaGetLastError();
+}
+
+// Voxels per lane and table entry: 2 K2, in chunks of 64 K2 along z.  An
+// entry costs about as much as one more pair of voxels (256^3 / 180 views,
+// ms for K2 = 1..4: 4.27, 3.13, 4.74, 2.64, i.e. 1.07, 1.56, 2.37, 2.64 per
+// chunk), so chunks x (K2 + 1) is what a grid costs.  9 bits of search
+// position hold a chunk's rays down to the pitch given here.
+int column_pairs(int nz, double pitch)
+{
+    static const double least[5] = {0, 0.26, 0.26, 0.42, 0.55};
+    int best = 1;
+    for (int k = 1; k <= 4; ++k)
+        if (pitch > least[k] && column_chunks(nz, k) * (k + 1) <= column_chunks(nz, best) * (best + 1)) best = k;
+    return best;
+}
+
+// Whether the column form is the faster adjoint: short z lines leave most of
+// a chunk's lanes idle (64^3: 37 us against 33 us for the warp-combined
+// scatter; 256^3: 2.64 ms against 4.37 ms), and with rays far apart most
+// voxels that it visits receive nothing.
+bool columns_pay(int nz, double pitch)
+{
+    const int k = column_pairs(nz, pitch);
+    return 33 * (k + 1) * column_chunks(nz, k) <= nz;
+}
+
+bool columns_pay(const ColumnForm &form, int nz) { return form.pitch_max <= 3.0 && columns_pay(nz, form.pitch); }
+
+// Adds A^T proj to vol.
+gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnForm &form, const gjp_geometry &g,
+                           float *vol, cudaStream_t s)
+{
+    const int K2 = column_pairs(V.n[2], form.pitch);
+    const int pad = line_pad(K2, form.pitch), nvp = line_length(g.nv, pad);
+    const size_t line_bytes = (size_t)g.nu * nvp * sizeof(float);
+    const int most = (int)std::max<size_t>(1, std::min<size_t>((size_t)g.n_views, (512ull << 20) / line_bytes));
+    void *ws = nullptr;
+    const gjp_status got = workspace_alloc((size_t)most * line_bytes + 256, s, &ws);
+    if (got != GJP_OK) return got;
+    ColumnJob j;
+    j.flag = static_cast<unsigned *>(ws);
+    float *lines = reinterpret_cast<float *>(static_cast<char *>(ws) + 256);
+    j.lines = lines;
+    j.V = V;
+    j.form = &form;
+    j.g = &g;
+    j.nvp = nvp;
+    j.pad = pad;
+    j.vol = vol;
+    j.s = s;
+    cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(unsigned), s);
+    for (int v0 = 0; v0 < g.n_views && e == cudaSuccess; v0 += most) {
+        j.view0 = v0;
+        j.n_views = std::min(most, g.n_views - v0);
+        const dim3 tg((unsigned)((g.nu + 31) / 32), (unsigned)((nvp + 31) / 32), (unsigned)j.n_views);
+        gjp_lines_kernel<<<tg, dim3(32, kTrRows), 0, s>>>(proj, V, form.d_cols, g.nu, g.nv, nvp, pad, v0, lines,
+                                                          static_cast<unsigned *>(ws));
+        if ((e = cudaGetLastError()) != cudaSuccess) break;
+        // View groups run one after another: their lines (the values, without
+        // the zeros) stay in the L2 while all tiles read them, 64 MB measured
+        // best (512^3, 216 views of 1 MB: 2 / 4 / 8 groups 38.3 / 38.0 /
+        // 39.2 ms per 360 views); small grids take more groups until every SM
+        // has some waves of warps, of eight views or more.
+        const double mb = (double)j.n_views * g.nu * g.nv * 4.0 / (64.0 * 1024 * 1024);
+        const double warps = 2.0 * V.n[0] * V.n[1] / kStrip * column_chunks(V.n[2], K2);
+        j.groups = std::max((int)std::ceil(mb), (int)std::ceil(10000.0 / warps));
+        j.groups = std::max(1, std::min(j.groups, (j.n_views + 7) / 8));
+        e = K2 == 4 ? launch_tiles<4>(j) : K2 == 3 ? launch_tiles<3>(j) : K2 == 2 ? launch_tiles<2>(j) : launch_tiles<1>(j);
+    }
+    const cudaError_t f = cudaFreeAsync(ws, s);
+    return e == cudaSuccess && f == cudaSuccess ? GJP_OK : GJP_ERR_CUDA;
+}
+
+}  // namespace gjp_detail

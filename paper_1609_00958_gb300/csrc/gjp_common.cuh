@@ -91,10 +91,45 @@ static_assert(4 * kBatch == 16, "the row-table march is written for 4-plane batc
 // limit as GJP_MIN_BLOCKS resident blocks of 4 warps
 constexpr int kMinBlocksMax = (GJP_MIN_BLOCKS * 4 + kMaxTileU - 1) / kMaxTileU;
 
+// Column form (gjp_columns.cu): scans whose detector rows run along z.
+// One detector column of one view: the (x, y) path its rays share and their
+// z positions, in fixed point (32 fraction bits; the pitch kPitchBits).
+struct Column {
+    long long Pa, Ga;       // transverse position on plane ic, increment per plane (as Ray)
+    long long Z0, Z1;       // z of the middle row on plane ic, increment per plane
+    long long Y0, Y1;       // z pitch per detector row on plane ic, increment per plane
+    int m, pad;             // driving axis (0 or 1)
+};
+// One view and driving axis m: source and direction in index units, which
+// give the detector column through a point of plane i, and the columns that
+// m drives.
+struct ColumnView {
+    float s_m, s_a, r0_m, ru_m, r0_a, ru_a;
+    int u_lo, u_hi;
+    int view, pad;
+};
+constexpr int kMaxColumns = 1 << 22;
+// Host: the views that each driving axis has columns of, and the least and
+// the largest row pitch (voxels).
+struct ColumnPlan {
+    std::vector<ColumnView> views[2];
+    double pitch = 0.0, pitch_max = 0.0;
+};
+// The column form on a device (one allocation, at d_views).
+struct ColumnForm {
+    enum State { kUnknown, kNone, kReady };
+    State state = kUnknown;
+    const ColumnView *d_views = nullptr;      // axis 0's, then axis 1's
+    Column *d_cols = nullptr;                 // [view][iu]
+    std::vector<int> view_ids[2];
+    double pitch = 0.0, pitch_max = 0.0;
+};
+
 struct gjp_cache_entry {
     int device;
     double key[9];
     ViewParams *d_table;
+    ColumnForm columns;
     int box_rows, box_cols4, box_cols8;   // slab box sizes for this grid (0 = not computed)
     void *tex = nullptr;                  // texture arrays of the texture families (gjp_texture.cu)
 };
@@ -198,6 +233,19 @@ inline int launch_view_group(const gjp_geometry &g, const int64_t n[3])
                       (int)std::min<int64_t>(n[2], INT_MAX)};
     return launch_view_group(g, m);
 }
+// Column form (gjp_columns.cu): whether g on this grid has it; the column
+// records; whether its adjoint is the faster one; A^T proj added to vol (errors of workspace_alloc, with nothing
+// queued, or GJP_ERR_CUDA).
+bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], const double o[3], ColumnPlan &plan);
+cudaError_t write_columns(const ViewParams *views, const VolParams &V, const gjp_geometry &g, Column *cols,
+                          cudaStream_t s);
+bool columns_pay(int nz, double pitch = 1.0);
+bool columns_pay(const ColumnForm &form, int nz);
+gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnForm &form, const gjp_geometry &g,
+                           float *vol, cudaStream_t s);
+// Stream-ordered workspace from the library's pool (gjp.cu): GJP_ERR_UNSUPPORTED
+// while s is being captured, GJP_ERR_OOM when there is no room.
+gjp_status workspace_alloc(size_t bytes, cudaStream_t s, void **out);
 // Tap-check faults recorded by the kernels of the other translation units
 // (debug build; 0 otherwise), read and cleared.
 unsigned batch_tap_faults();
@@ -534,7 +582,8 @@ __device__ __forceinline__ void plane_interval(long long P, long long G, int ic,
 // two roots of a quadratic (float32; a sample within ~1e-4 plane of the
 // circle may fall on either side, which cannot matter for a volume that is
 // zero near the cylinder wall, the setting this option is for).
-__device__ __forceinline__ void clip_to_fov(const VolParams &V, Ray &R, int m)
+__device__ __forceinline__ void fov_planes(const VolParams &V, int m, int ic, long long Pa, long long Ga, long long Pb,
+                                           long long Gb, int &lo, int &hi)
 {
     const float inv = 2.3283064365386963e-10f;   // 2^-32
     // index position at t = 0 and per plane, for x and y
@@ -542,13 +591,12 @@ __device__ __forceinline__ void clip_to_fov(const VolParams &V, Ray &R, int m)
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const bool is_m = k == m, is_a = k == ((m == 0) ? 1 : 0);
-        p0[k] = is_m ? (float)R.ic : __ll2float_rn(is_a ? R.Pa : R.Pb) * inv;
-        dp[k] = is_m ? 1.0f : __ll2float_rn(is_a ? R.Ga : R.Gb) * inv;
+        p0[k] = is_m ? (float)ic : __ll2float_rn(is_a ? Pa : Pb) * inv;
+        dp[k] = is_m ? 1.0f : __ll2float_rn(is_a ? Ga : Gb) * inv;
     }
     const float X0 = V.h[0] * (p0[0] - 0.5f * (float)(V.n[0] - 1)), dX = V.h[0] * dp[0];
     const float Y0 = V.h[1] * (p0[1] - 0.5f * (float)(V.n[1] - 1)), dY = V.h[1] * dp[1];
     const float A = dX * dX + dY * dY, B = X0 * dX + Y0 * dY, C = X0 * X0 + Y0 * Y0 - V.fov_r2;
-    int lo, hi;
     if (A <= 0.0f) {                       // no motion in (x, y): all planes or none
         lo = C <= 0.0f ? 0 : 1;
         hi = C <= 0.0f ? 0x3fffffff : 0;
@@ -560,10 +608,16 @@ __device__ __forceinline__ void clip_to_fov(const VolParams &V, Ray &R, int m)
         } else {
             const float sq = sqrtf(disc);
             const float t1 = (-B - sq) / A, t2 = (-B + sq) / A;
-            lo = R.ic + (int)ceilf(fmaxf(t1, -1.0e9f));
-            hi = R.ic + (int)floorf(fminf(t2, 1.0e9f));
+            lo = ic + (int)ceilf(fmaxf(t1, -1.0e9f));
+            hi = ic + (int)floorf(fminf(t2, 1.0e9f));
         }
     }
+}
+
+__device__ __forceinline__ void clip_to_fov(const VolParams &V, Ray &R, int m)
+{
+    int lo, hi;
+    fov_planes(V, m, R.ic, R.Pa, R.Ga, R.Pb, R.Gb, lo, hi);
     R.s_lo = max(R.s_lo, lo);
     R.s_hi = min(R.s_hi, hi);
     R.j_lo = max(R.j_lo, lo);
