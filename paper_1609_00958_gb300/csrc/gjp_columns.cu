@@ -135,14 +135,17 @@ __global__ void gjp_columns_kernel(const ViewParams *__restrict__ views, VolPara
     setup_ray(vp, V, (float)u - 0.5f * (float)(nu - 1), 0.0f, R);
     const int m = R.m, a = 1 - m;
     const float fu = (float)u - 0.5f * (float)(nu - 1);
-    const f2 rm = m == 0 ? f2_affine(vp.rh, vp.rl, 0, fu, 0.0f) : f2_affine(vp.rh, vp.rl, 1, fu, 0.0f);
+    const auto lateral = [&](int k) {
+        return f2_affine({vp.rh[k], vp.rl[k]}, {vp.rh[3 + k], vp.rl[3 + k]}, {vp.rh[6 + k], vp.rl[6 + k]}, fu, 0.0f);
+    };
+    const f2 rm = m == 0 ? lateral(0) : lateral(1);
+    const float inv = __fdividef(1.0f, rm.hi);
     const f2 mv = {a == 0 ? vp.mh[6] : vp.mh[7], a == 0 ? vp.ml[6] : vp.ml[7]};   // dL_a / dv
-    f2 dq = f2_div(mv, rm);
+    f2 dq = f2_div(mv, rm, inv);
     if (2 == (m + 1) % 3) dq = f2_neg(dq);
-    const f2 dg = f2_div({vp.rh[8], vp.rl[8]}, rm);                                 // d(rt_z) / dv
+    const f2 dg = f2_div({vp.rh[8], vp.rl[8]}, rm, inv);                            // d(rt_z) / dv
     const int nm = m == 0 ? V.n[0] : V.n[1];
-    const float delta = (float)R.ic - 0.5f * (float)(nm - 1);
-    const f2 y0 = f2_add(dq, f2_mul_f(dg, delta));
+    const f2 y0 = f2_shift(dq, 0.0f, dg, (float)R.ic - 0.5f * (float)(nm - 1));
     const float scale = 1099511627776.0f;   // 2^kPitchBits
     Column c;
     c.Pa = R.Pa;

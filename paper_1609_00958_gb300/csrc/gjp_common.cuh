@@ -30,7 +30,7 @@ namespace gjp_detail {
 // Per-view device record: FP64 host quantities (index units; pixel
 // coordinates centred on the panel, u = iu - (nu-1)/2, v = iv - (nv-1)/2)
 // split into hi + lo FP32 parts.
-struct ViewParams {
+struct __align__(16) ViewParams {
     float rh[9], rl[9];  // R0[3], RU[3], RV[3]: ray direction d - s (Eq. 2)
     float mh[9], ml[9];  // M0[3], MU[3], MV[3]: moment (s - c) x r about the centre c
 };
@@ -272,40 +272,37 @@ __device__ __forceinline__ f2 quick_two_sum(float a, float b)  // |a| >= |b|
     return {s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
-__device__ __forceinline__ f2 f2_add(f2 x, f2 y)
+// x0 + u xu + v xv: the leading products and sums are exact (pairs), their
+// tails are added in FP32, so the result is good to about 2^-46 of its
+// largest term.
+__device__ __forceinline__ f2 f2_affine(f2 x0, f2 xu, f2 xv, float u, float v)
 {
-    f2 s = two_sum(x.hi, y.hi);
-    const f2 t = two_sum(x.lo, y.lo);
-    s.lo = __fadd_rn(s.lo, t.hi);
-    s = quick_two_sum(s.hi, s.lo);
-    s.lo = __fadd_rn(s.lo, t.lo);
-    return quick_two_sum(s.hi, s.lo);
+    const float p = __fmul_rn(xu.hi, u), q = __fmul_rn(xv.hi, v);
+    const f2 s = two_sum(x0.hi, p), t = two_sum(s.hi, q);
+    float lo = __fmaf_rn(xu.lo, u, __fmaf_rn(xu.hi, u, -p));
+    lo = __fadd_rn(lo, __fmaf_rn(xv.lo, v, __fmaf_rn(xv.hi, v, -q)));
+    lo = __fadd_rn(__fadd_rn(lo, x0.lo), __fadd_rn(s.lo, t.lo));
+    return quick_two_sum(t.hi, lo);
 }
 
-__device__ __forceinline__ f2 f2_mul_f(f2 x, float f)
+// x / y for a float `inv` within a few units in the last place of 1 / y.hi:
+// quotient, remainder (one FMA) and the remainder's quotient; good to about
+// 2^-44 of the result.
+__device__ __forceinline__ f2 f2_div(f2 x, f2 y, float inv)
 {
-    const float p = __fmul_rn(x.hi, f);
-    float e = __fmaf_rn(x.hi, f, -p);
-    e = __fmaf_rn(x.lo, f, e);
-    return quick_two_sum(p, e);
+    const float q = __fmul_rn(x.hi, inv);
+    const float r = __fadd_rn(__fmaf_rn(-q, y.hi, x.hi), __fmaf_rn(-q, y.lo, x.lo));
+    return quick_two_sum(q, __fmul_rn(r, inv));
 }
 
-__device__ __forceinline__ f2 f2_div(f2 x, f2 y)
+// q + c + g d as an unnormalised pair (c and g d exact)
+__device__ __forceinline__ f2 f2_shift(f2 q, float c, f2 g, float d)
 {
-    const float q1 = __fdiv_rn(x.hi, y.hi);
-    const f2 r = f2_add(x, f2_mul_f(y, -q1));
-    const float q2 = __fdiv_rn(r.hi, y.hi);
-    return quick_two_sum(q1, q2);
+    const f2 s = two_sum(q.hi, c), t = two_sum(s.hi, __fmul_rn(g.hi, d));
+    return {t.hi, __fadd_rn(__fmaf_rn(g.lo, d, q.lo), __fadd_rn(s.lo, t.lo))};
 }
 
 __device__ __forceinline__ f2 f2_neg(f2 x) { return {-x.hi, -x.lo}; }
-
-// X0[k] + u XU[k] + v XV[k] from a hi/lo coefficient block of 9 floats.
-__device__ __forceinline__ f2 f2_affine(const float *h, const float *l, int k, float u, float v)
-{
-    const f2 x0 = {h[k], l[k]}, xu = {h[3 + k], l[3 + k]}, xv = {h[6 + k], l[6 + k]};
-    return f2_add(f2_add(x0, f2_mul_f(xu, u)), f2_mul_f(xv, v));
-}
 
 // round(x * 2^32) as a 64-bit fixed-point number (|x| < 2^30).
 __device__ __forceinline__ long long f2_to_fixed(f2 x)
@@ -544,34 +541,49 @@ __device__ __forceinline__ long long pos_at(long long P, long long G, int i, int
     return P + (long long)(i - ic) * G;
 }
 
-// Planes i in [0, nm - 1] with lo < P + (i - ic) G < hi (fixed point,
-// strict).  A float estimate brackets the crossings; the exact integer test
-// then trims the bracket (positions are monotone in i).
-__device__ __forceinline__ void plane_interval(long long P, long long G, int ic, long long lo, long long hi,
-                                               int nm, int &a, int &b)
+// The first plane i in [0, nm] with P + (i - ic) G > lo, for G > 0 and inv
+// near 1 / G (fixed point; nm when there is none): a float estimate, which is
+// rarely a plane off, moved to the exact place by the loop's own integer
+// arithmetic.
+__device__ __forceinline__ int first_above(long long P, long long G, float inv, int ic, long long lo, int nm)
 {
+    const float x = floorf(__ll2float_rn(lo - P) * inv);
+    int i = ic + 1 + (int)fminf(fmaxf(x, (float)(-1 - ic)), (float)(nm - ic));
+    i = min(max(i, 0), nm);
+    long long p = pos_at(P, G, i, ic);
+    while (i > 0 && p - G > lo) {
+        --i;
+        p -= G;
+    }
+    while (i < nm && p <= lo) {
+        ++i;
+        p += G;
+    }
+    return i;
+}
+
+// Planes s0 .. s1 of one transverse axis of n points on which a sample can
+// have a non-zero tap (-1 < p < n), and planes j0 .. j1 on which both its
+// taps lie in the grid (0 <= p < n - 1); positions are monotone in i.
+__device__ __forceinline__ void plane_ranges(long long P, long long G, int ic, int n, int nm, int &s0, int &s1, int &j0,
+                                             int &j1)
+{
+    const long long one = 1LL << 32, top = (long long)n * one;
     if (G == 0) {
-        const bool in = lo < P && P < hi;
-        a = 0;
-        b = in ? nm - 1 : -1;
+        s0 = j0 = 0;
+        s1 = -one < P && P < top ? nm - 1 : -1;
+        j1 = 0 <= P && P < top - one ? nm - 1 : -1;
         return;
     }
-    const float g = __ll2float_rn(G);
-    const float t1 = __ll2float_rn(lo - P) / g, t2 = __ll2float_rn(hi - P) / g;
-    const float lim = 3.0e7f;
-    const float tmin = fmaxf(fminf(t1, t2), -lim), tmax = fminf(fmaxf(t1, t2), lim);
-    a = max(0, ic + (int)floorf(tmin) - 2);
-    b = min(nm - 1, ic + (int)ceilf(tmax) + 2);
-    while (a <= b) {
-        const long long p = pos_at(P, G, a, ic);
-        if (lo < p && p < hi) break;
-        ++a;
-    }
-    while (b >= a) {
-        const long long p = pos_at(P, G, b, ic);
-        if (lo < p && p < hi) break;
-        --b;
-    }
+    // a falling position is a rising one seen from the other end of the axis
+    const bool up = G > 0;
+    const long long Q = up ? P : -P, g = up ? G : -G;
+    const float inv = __fdividef(1.0f, __ll2float_rn(g));
+    // p > -1, p >= 0, p >= n - 1, p >= n (rising), or -p > -n, > 1 - n, > -1 ... (falling)
+    s0 = first_above(Q, g, inv, ic, up ? -one : -top, nm);
+    j0 = first_above(Q, g, inv, ic, up ? -1 : one - top, nm);
+    j1 = first_above(Q, g, inv, ic, up ? top - one - 1 : 0, nm) - 1;
+    s1 = first_above(Q, g, inv, ic, up ? top - 1 : one - 1, nm) - 1;
 }
 
 // Field-of-view cylinder (the speed section samples each ray only on its
@@ -626,25 +638,28 @@ __device__ __forceinline__ void clip_to_fov(const VolParams &V, Ray &R, int m)
 
 __device__ __forceinline__ void setup_ray(const ViewParams &vp, const VolParams &V, float u, float v, Ray &R)
 {
-    const f2 r0 = f2_affine(vp.rh, vp.rl, 0, u, v);
-    const f2 r1 = f2_affine(vp.rh, vp.rl, 1, u, v);
-    const f2 r2 = f2_affine(vp.rh, vp.rl, 2, u, v);
+    const auto r_at = [&](int k) {
+        return f2_affine({vp.rh[k], vp.rl[k]}, {vp.rh[3 + k], vp.rl[3 + k]}, {vp.rh[6 + k], vp.rl[6 + k]}, u, v);
+    };
+    const f2 r0 = r_at(0), r1 = r_at(1), r2 = r_at(2);
     int m = 0;                                           // Eq. 3, ties to the lowest index
     if (fabsf(r1.hi) > fabsf(r0.hi)) m = 1;
     if (fabsf(r2.hi) > fabsf(sel3(r0.hi, r1.hi, r2.hi, m))) m = 2;
     const int a = (m == 0) ? 1 : 0;
     const int b = (m == 2) ? 1 : 2;
-    const f2 rm = sel3(r0, r1, r2, m), ra = sel3(r0, r1, r2, a), rb = sel3(r0, r1, r2, b);
+    const f2 rm = sel3(r0, r1, r2, m), ra = a == 0 ? r0 : r1, rb = b == 1 ? r1 : r2;
     // moment components L_a, L_b: the centre-plane crossing is
     // q_a = -+ L_b / r_m, q_b = -+ L_a / r_m  (minus for the cyclic order (m, k, j))
-    const f2 L0 = f2_affine(vp.mh, vp.ml, 0, u, v);
-    const f2 L1 = f2_affine(vp.mh, vp.ml, 1, u, v);
-    const f2 L2 = f2_affine(vp.mh, vp.ml, 2, u, v);
-    const f2 La = sel3(L0, L1, L2, a), Lb = sel3(L0, L1, L2, b);
-    f2 qa = f2_div(Lb, rm), qb = f2_div(La, rm);
+    const auto moment = [&](bool first, int k0, int k1) {   // component k0 or k1
+        const auto c = [&](int j) { return f2{first ? vp.mh[j + k0] : vp.mh[j + k1], first ? vp.ml[j + k0] : vp.ml[j + k1]}; };
+        return f2_affine(c(0), c(3), c(6), u, v);
+    };
+    const f2 La = moment(a == 0, 0, 1), Lb = moment(b == 1, 1, 2);
+    const float inv = __fdividef(1.0f, rm.hi);
+    f2 qa = f2_div(Lb, rm, inv), qb = f2_div(La, rm, inv);
     if (a == (m + 1) % 3) qa = f2_neg(qa);
     if (b == (m + 1) % 3) qb = f2_neg(qb);
-    const f2 ga = f2_div(ra, rm), gb = f2_div(rb, rm);   // Eq. 4
+    const f2 ga = f2_div(ra, rm, inv), gb = f2_div(rb, rm, inv);   // Eq. 4
 
     const int nm = sel3(V.n[0], V.n[1], V.n[2], m);
     R.m = m;
@@ -657,23 +672,17 @@ __device__ __forceinline__ void setup_ray(const ViewParams &vp, const VolParams 
     const float cm = 0.5f * (float)(nm - 1);
     R.ic = (nm - 1) >> 1;                                 // floor(c_m)
     const float delta = (float)R.ic - cm;                 // 0 or -1/2
-    const f2 Pa = f2_add(f2_add(qa, {0.5f * (float)(R.na - 1), 0.0f}), f2_mul_f(ga, delta));
-    const f2 Pb = f2_add(f2_add(qb, {0.5f * (float)(R.nb - 1), 0.0f}), f2_mul_f(gb, delta));
-    R.Pa = f2_to_fixed(Pa);
-    R.Pb = f2_to_fixed(Pb);
+    R.Pa = f2_to_fixed(f2_shift(qa, 0.5f * (float)(R.na - 1), ga, delta));
+    R.Pb = f2_to_fixed(f2_shift(qb, 0.5f * (float)(R.nb - 1), gb, delta));
     R.Ga = f2_to_fixed(ga);
     R.Gb = f2_to_fixed(gb);
     const float hm = sel3(V.h[0], V.h[1], V.h[2], m);
     const float ha = sel3(V.h[0], V.h[1], V.h[2], a) * ga.hi, hb = sel3(V.h[0], V.h[1], V.h[2], b) * gb.hi;
     R.step = sqrtf(hm * hm + ha * ha + hb * hb);
 
-    // support: -1 < p < n on both transverse axes; interior: 0 <= p < n - 1
-    const long long one = 1LL << 32;
     int sa0, sa1, sb0, sb1, ja0, ja1, jb0, jb1;
-    plane_interval(R.Pa, R.Ga, R.ic, -one, (long long)R.na * one, nm, sa0, sa1);
-    plane_interval(R.Pb, R.Gb, R.ic, -one, (long long)R.nb * one, nm, sb0, sb1);
-    plane_interval(R.Pa, R.Ga, R.ic, -1, (long long)(R.na - 1) * one, nm, ja0, ja1);
-    plane_interval(R.Pb, R.Gb, R.ic, -1, (long long)(R.nb - 1) * one, nm, jb0, jb1);
+    plane_ranges(R.Pa, R.Ga, R.ic, R.na, nm, sa0, sa1, ja0, ja1);
+    plane_ranges(R.Pb, R.Gb, R.ic, R.nb, nm, sb0, sb1, jb0, jb1);
     R.s_lo = max(sa0, sb0);
     R.s_hi = min(sa1, sb1);
     R.j_lo = max(max(ja0, jb0), R.s_lo);
@@ -683,10 +692,19 @@ __device__ __forceinline__ void setup_ray(const ViewParams &vp, const VolParams 
 
 __device__ __forceinline__ void load_view(const ViewParams *__restrict__ views, int k, ViewParams &vp)
 {
-    const float *src = reinterpret_cast<const float *>(views + k);
+    static_assert(sizeof(ViewParams) == 9 * sizeof(float4), "a view's record is read in 16-byte words");
+    const float4 *src = reinterpret_cast<const float4 *>(views + k);
+    float4 w[9];
+#pragma unroll
+    for (int j = 0; j < 9; ++j) w[j] = __ldg(src + j);
     float *dst = reinterpret_cast<float *>(&vp);
 #pragma unroll
-    for (int j = 0; j < 36; ++j) dst[j] = __ldg(src + j);
+    for (int j = 0; j < 9; ++j) {
+        dst[4 * j] = w[j].x;
+        dst[4 * j + 1] = w[j].y;
+        dst[4 * j + 2] = w[j].z;
+        dst[4 * j + 3] = w[j].w;
+    }
 }
 
 // Boundary planes: the support planes outside the interior range, visited
