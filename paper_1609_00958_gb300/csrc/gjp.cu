@@ -288,6 +288,28 @@ const ColumnForm *get_columns(const gjp_geometry *gc, gjp_cache_entry &e, const 
     }
 }
 
+// The same with more loads in flight per warp and fewer warps: 8 planes of
+// the row-table march per load batch (from a z-paired copy 16), at 20 (16)
+// warps per SM instead of 32.  For launches whose taps mostly come from DRAM
+// or a cold L2, which wait for latency (deep_loads); bit for bit the same
+// sums.
+template <bool PAIRS> constexpr int kDeepPlanes = PAIRS ? 16 : 8;
+template <typename T, bool SPL, bool PAIRS>
+__global__ void __launch_bounds__(kTileV * kTileU, PAIRS ? 4 : 5) gjp_forward_deep_kernel(
+    const T *__restrict__ vol, VolParams V, const ViewParams *__restrict__ views,
+    int nu, int nv, int n_tv, int n_views, int view_group, float *__restrict__ proj,
+    const typename PairOf<T>::type *__restrict__ pairs)
+{
+    int tile, view;
+    block_tile_view(n_views, view_group, tile, view);
+    const int iv = (tile % n_tv) * kTileV + threadIdx.x;
+    const int iu = (tile / n_tv) * (int)blockDim.y + threadIdx.y;
+    const unsigned act = __ballot_sync(0xffffffffu, iv < nv && iu < nu);
+    if (iv >= nv || iu >= nu) return;
+    proj[((size_t)view * nv + iv) * nu + iu] =
+        forward_ray<T, int, SPL, PAIRS, kDeepPlanes<PAIRS>>(vol, V, views + view, nu, nv, iu, iv, act, (int)threadIdx.y, pairs);
+}
+
 template <typename T, typename Index, bool SPL, bool PAIRS>
 __global__ void __launch_bounds__(kMaxThreads, kMinBlocksMax) gjp_forward_kernel(
     const T *__restrict__ vol, VolParams V, const ViewParams *__restrict__ views,
@@ -1638,6 +1660,30 @@ cudaError_t launch_gather_pf(const T *vol, gjp_dtype dt, const int64_t n[3], con
     return cudaGetLastError();
 }
 
+// Whether a launch takes the kernel with deeper load batches.  Its taps come
+// from the L2 as far as the views of a group (n_views, group) share them and
+// the volume outlives the 129 MB L2.  Measured, default -> deep (ms; views x
+// step between them):
+//   float32: 512^3, 360 x 1 deg 35.15 -> 35.35, 48 x 1 deg 4.51 -> 4.52,
+//     48 x 2 deg (groups of 8) 4.87 -> 4.78, 48 x 7.5 deg 6.33 -> 5.64;
+//     768^3, 36 x 0.5 deg (14) 11.0 -> 10.6, 36 x 3 deg 15.3 -> 13.5;
+//     1024^3, 32 x 0.5 deg (8) 25.4 -> 23.0, 32 x 3 deg 40.0 -> 32.7;
+//     256^3, 64 views 0.83 -> 0.85, 16 views 0.239 -> 0.232, one 0.061 -> 0.034;
+//     128^3, 16 views 0.0464 -> 0.0448.
+//   16-bit, z-paired: 512^3, 360 x 1 deg 31.6 -> 33.0, 48 x 2 deg (8) 4.46 -> 4.58,
+//     48 x 4 deg (4) 4.74 -> 4.73, 48 x 7.5 deg (2) 5.48 -> 5.06; 768^3, 36 x
+//     0.5 deg (14) 10.26 -> 10.25, 36 x 1 deg (7) 11.2 -> 10.8; 1024^3, 32 x 0.5 deg
+//     (8) 22.7 -> 21.0, 60 x 6 deg 61.6 -> 53.0; 256^3 always slower.
+//   16-bit, from the volume: 512^3, 16 views 1.89 -> 1.84, 4 views 0.631 -> 0.573;
+//     256^3, 8 views 0.137 -> 0.136, 16 views 0.243 -> 0.248.
+bool deep_loads(const int n[3], int n_views, int group, bool f32, bool pairs)
+{
+    const double voxels = (double)n[0] * n[1] * n[2];
+    if (f32) return n_views <= 16 || (voxels >= 1.0e8 && group < 16);
+    if (pairs) return (voxels >= 2.6e8 && group < 16) || (voxels >= 6.7e7 && group <= 3);
+    return n_views <= 8 || (voxels >= 6.7e7 && n_views < 32);
+}
+
 // pairs: the z-paired copy of vol for the row-table march (32-bit offsets
 // only), or null to read the taps from vol.
 template <typename T>
@@ -1652,6 +1698,19 @@ cudaError_t launch_gather_shaped(const T *vol, const VolParams &V, const ViewPar
     const bool spl = sh.spl;
     const int nu = sh.nu, nv = sh.nv, nvw = sh.n_views, vgp = sh.view_group;
     const size_t rows = (size_t)sh.tile_u * 32 * sizeof(uint2);   // row tables (32-bit offsets only)
+    if (i32 && sh.tile_u <= kTileU && !(pairs && std::is_same<T, float>::value) &&
+        deep_loads(V.n, nvw, vgp, std::is_same<T, float>::value, pairs != nullptr)) {
+        if constexpr (!std::is_same<T, float>::value) {
+            if (pairs) {
+                auto kern = spl ? gjp_forward_deep_kernel<T, true, true> : gjp_forward_deep_kernel<T, false, true>;
+                kern<<<grid, block, rows, s>>>(vol, V, table, nu, nv, n_tv, nvw, vgp, proj, pairs);
+                return cudaGetLastError();
+            }
+        }
+        auto kern = spl ? gjp_forward_deep_kernel<T, true, false> : gjp_forward_deep_kernel<T, false, false>;
+        kern<<<grid, block, rows, s>>>(vol, V, table, nu, nv, n_tv, nvw, vgp, proj, pairs);
+        return cudaGetLastError();
+    }
 #define GJP_LAUNCH_FWD(I, S, P, SMEM)                                                                              \
     gjp_forward_kernel<T, I, S, P><<<grid, block, SMEM, s>>>(vol, V, table, nu, nv, n_tv, nvw, vgp, proj, pairs)
     if (i32 && pairs) {

@@ -940,7 +940,7 @@ __device__ __forceinline__ float2 rows_block(const S *__restrict__ src, const ui
 // `rows` is this warp's 32-entry table (256 bytes, 16-byte aligned): per
 // pair of planes the row weight bits of both, then the row offsets of both
 // (the layout rows_block reads).
-template <typename T, bool SPL, typename S>
+template <typename T, bool SPL, int B, typename S>
 __device__ __forceinline__ float march_interior_rows(const S *__restrict__ src, const Ray &R, bool rev,
                                                      uint4 *__restrict__ rows, int lane)
 {
@@ -981,10 +981,10 @@ __device__ __forceinline__ float march_interior_rows(const S *__restrict__ src, 
             const int k = w + kb;
             const int ip = i0 + dir * k;
             if (k >= K0 && k + 15 <= K1)              // warp-uniform
-                acc = __fadd2_rn(acc, rows_block<T, SPL, false, kRowBatch<S>>(src, rows + kb / 2, pb, gb, sa, 0, 0, 16,
+                acc = __fadd2_rn(acc, rows_block<T, SPL, false, B>(src, rows + kb / 2, pb, gb, sa, 0, 0, 16,
                                                                              ip, dir, R));
             else
-                acc = __fadd2_rn(acc, rows_block<T, SPL, true, kRowBatch<S>>(src, rows + kb / 2, pb, gb, sa, k - k_lo, cnt, L - k,
+                acc = __fadd2_rn(acc, rows_block<T, SPL, true, B>(src, rows + kb / 2, pb, gb, sa, k - k_lo, cnt, L - k,
                                                                ip, dir, R));
         }
     }
@@ -1010,8 +1010,9 @@ __device__ __forceinline__ int lane_id()
 // whose table entry is *view (Algorithm 1).  Called by every lane of the
 // warp set in `act` (the lanes that hold a ray; they share the warp-level
 // choice of march direction).  PAIRS: the row-table march reads its taps
-// from `pairs`, the z-paired copy of vol (32-bit offsets only).
-template <typename T, typename Index, bool SPL, bool PAIRS = false>
+// from `pairs`, the z-paired copy of vol (32-bit offsets only).  DEEP: planes
+// per load batch of the row-table march (0: the default).
+template <typename T, typename Index, bool SPL, bool PAIRS = false, int DEEP = 0>
 __device__ __forceinline__ float forward_ray(const T *__restrict__ vol, const VolParams &V,
                                              const ViewParams *__restrict__ view, int nu, int nv, int iu, int iv,
                                              unsigned act, int rows_slot = -1,
@@ -1042,8 +1043,9 @@ __device__ __forceinline__ float forward_ray(const T *__restrict__ vol, const Vo
             const long long Pa0 = __shfl_sync(act, R.Pa, 0), Ga0 = __shfl_sync(act, R.Ga, 0);
             if (__all_sync(act, R.m == m0 && R.Pa == Pa0 && R.Ga == Ga0) && m0 != 2) {
                 uint4 *rows = gjp_row_tables + 16 * rows_slot;
-                const float acc = PAIRS ? march_interior_rows<T, SPL>(pairs, R, rev, rows, lane_id())
-                                        : march_interior_rows<T, SPL>(vol, R, rev, rows, lane_id());
+                using P = typename PairOf<T>::type;
+                const float acc = PAIRS ? march_interior_rows<T, SPL, DEEP ? DEEP : kRowBatch<P>>(pairs, R, rev, rows, lane_id())
+                                        : march_interior_rows<T, SPL, DEEP ? DEEP : kRowBatch<T>>(vol, R, rev, rows, lane_id());
                 return (acc + bsum) * R.step;
             }
         }
