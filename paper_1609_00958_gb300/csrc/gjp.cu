@@ -1070,6 +1070,79 @@ __device__ __forceinline__ void combine_march(const Ray &R, int I0, int I1, int 
         combine_plane<Index, SPL, true, CLIP, RUNS, ASC>(R, i, yw, pa, pb, plane, sa, na, nb, vol);
 }
 
+// Warps without a common row whose rays still follow one another along z (a
+// detector tilted against the rotation axis): neighbouring rays mostly land
+// on the same row of a plane, one voxel apart, and then the lower ray's two
+// upper taps join the next ray's lower taps as above.  Every lane steps its
+// own row.  192^3 / 96 views with a detector tilted by 0.7 degrees: 2.73 ms
+// tap by tap, 1.48 ms so (2.4 reductions per sample instead of 4).
+template <typename Index, bool SPL, bool CHECKED, bool CLIP, bool ASC>
+__device__ __forceinline__ void skew_planes(const Ray &R, int i, int i_end, float yw, float *__restrict__ vol)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x;
+    const bool has_prev = ASC ? lane > 0 : lane < 31, has_next = ASC ? lane < 31 : lane > 0;
+    const auto from_prev = [full](auto v) { return ASC ? __shfl_up_sync(full, v, 1) : __shfl_down_sync(full, v, 1); };
+    const Index sa = (Index)R.sa, sm = (Index)R.sm;
+    const unsigned na = (unsigned)R.na, nb = (unsigned)R.nb;
+    unsigned long long pa = (unsigned long long)pos_at(R.Pa, R.Ga, i, R.ic);
+    unsigned long long pb = (unsigned long long)pos_at(R.Pb, R.Gb, i, R.ic);
+    Index plane = (Index)i * sm;
+    for (; i <= i_end; ++i) {
+        const int ia = floor_of(pa), ib = floor_of(pb);
+        const float da = upper_weight<SPL>(frac_of(pa)), db = upper_weight<SPL>(frac_of(pb));
+        const float yi = (!CLIP || (i >= R.s_lo && i <= R.s_hi)) ? yw : 0.0f;
+        const float y1 = yi * da, y0 = __fmaf_rn(-yi, da, yi);        // to rows ia + 1 and ia
+        const float t01 = y0 * db, t11 = y1 * db;                     // upper z taps
+        float t00 = __fmaf_rn(-y0, db, y0), t10 = __fmaf_rn(-y1, db, y1);
+        const Index off = plane + (Index)ia * sa + (Index)ib;
+        const Index off_p = from_prev(off);
+        const float t01_p = from_prev(t01), t11_p = from_prev(t11);
+        const bool take = has_prev && off_p + 1 == off;
+        if (take) {
+            t00 += t01_p;
+            t10 += t11_p;
+        }
+        const unsigned takes = __ballot_sync(full, take);
+        const bool taken = has_next && ((ASC ? takes >> 1 : takes << 1) >> lane & 1u);
+        float *p = vol + off;
+        const bool w0 = t00 != 0.0f || t10 != 0.0f, w1 = !taken && yi != 0.0f;
+        if (CHECKED) {
+            const bool r0 = (unsigned)ia < na, r1 = (unsigned)(ia + 1) < na;   // zero border
+            const bool z0 = (unsigned)ib < nb, z1 = (unsigned)(ib + 1) < nb;
+            red_add_if(w0 && r0 && z0, p, t00);
+            red_add_if(w0 && r1 && z0, p + sa, t10);
+            red_add_if(w1 && r0 && z1, p + 1, t01);
+            red_add_if(w1 && r1 && z1, p + sa + 1, t11);
+        } else {
+            const bool ok = taps_in_grid(i, ia, ib, R.nm, R.na, R.nb);   // always true but in the debug build
+            red_add2_if(ok && w0, p, t00, p + sa, t10);
+            red_add2_if(ok && w1, p + 1, t01, p + sa + 1, t11);
+        }
+        pa += (unsigned long long)R.Ga;
+        pb += (unsigned long long)R.Gb;
+        plane += sm;
+    }
+}
+
+// All planes of such a warp: those interior for every lane unchecked.
+template <typename Index, bool SPL, bool CLIP, bool ASC>
+__device__ __forceinline__ void skew_march(const Ray &R, float ys, float *__restrict__ vol)
+{
+    const unsigned full = 0xffffffffu;
+    const bool act = ys != 0.0f && R.s_lo <= R.s_hi;
+    const int I0 = __reduce_min_sync(full, act ? R.s_lo : INT_MAX), I1 = __reduce_max_sync(full, act ? R.s_hi : -1);
+    const int F0 = max(I0, __reduce_max_sync(full, R.j_lo)), F1 = min(I1, __reduce_min_sync(full, R.j_hi));
+    const float yw = act ? ys : 0.0f;
+    if (F0 > F1) {
+        skew_planes<Index, SPL, true, CLIP, ASC>(R, I0, I1, yw, vol);
+        return;
+    }
+    skew_planes<Index, SPL, true, CLIP, ASC>(R, I0, F0 - 1, yw, vol);
+    skew_planes<Index, SPL, false, false, ASC>(R, F0, F1, yw, vol);
+    skew_planes<Index, SPL, true, CLIP, ASC>(R, F1 + 1, I1, yw, vol);
+}
+
 template <typename Index, bool SPL, bool CLIP>
 __global__ void __launch_bounds__(kMaxThreads) gjp_adjoint_combine_kernel(
     const float *__restrict__ proj, VolParams V, const ViewParams *__restrict__ views,
@@ -1101,7 +1174,19 @@ __global__ void __launch_bounds__(kMaxThreads) gjp_adjoint_combine_kernel(
     constexpr bool USE_ROWS = GJP_ROWS && std::is_same<Index, int>::value;
     uint2 *rows = row_table(threadIdx.y);
     if (!uniform) {
-        if (ys != 0.0f) scatter_ray<Index, SPL>(R, ys, vol);
+        // rays one after another along z on the centre plane, a third of a
+        // voxel to 1.7 voxels apart, and less than half a voxel apart across
+        // (z lines shorter than 4 voxels: a row's end could pass for the
+        // next row's start)
+        const long long one = 1LL << 32;
+        const long long za = __shfl_down_sync(full, R.Pa, 1) - R.Pa, zb = __shfl_down_sync(full, R.Pb, 1) - R.Pb;
+        const bool last = lane == 31;
+        const bool row = R.m == m0 && m0 != 2 && R.nb >= 4 && (last || (2 * za < one && -2 * za < one));
+        const bool up = __all_sync(full, row && (last || (3 * zb > one && 10 * zb < 17 * one)));
+        const bool down = __all_sync(full, row && (last || (-3 * zb > one && -10 * zb < 17 * one)));
+        if (up) skew_march<Index, SPL, CLIP, true>(R, ys, vol);
+        else if (down) skew_march<Index, SPL, CLIP, false>(R, ys, vol);
+        else if (ys != 0.0f) scatter_ray<Index, SPL>(R, ys, vol);
         return;
     }
     const bool act = ys != 0.0f && R.s_lo <= R.s_hi;
