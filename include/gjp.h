@@ -164,9 +164,9 @@ gjp_status gjp_forward(const void *d_volume, gjp_dtype dtype, int64_t nx, int64_
 
 /* Kernel family used by gjp_forward_ex. */
 typedef enum {
-    GJP_PATH_AUTO = 0,   /* the library's fastest family for the call (forward: PAIRS for
-                            16-bit storage over 32 or more views and 2^27 view-voxels
-                            where it applies, else GATHER; adjoint: COMBINE) */
+    GJP_PATH_AUTO = 0,   /* the library's fastest family for the call (forward: the column
+                            form where it applies, else PAIRS for 16-bit storage over 32
+                            or more views and 2^27 view-voxels, else GATHER; adjoint: COMBINE) */
     GJP_PATH_GATHER = 1, /* one thread per ray, taps gathered from global memory */
     GJP_PATH_SLAB = 2,   /* detector tiles stream per-plane voxel boxes into shared memory
                             with TMA; needs a 16-byte aligned volume whose z row is a
@@ -205,6 +205,16 @@ typedef enum {
  * near 1e-4 .. 1e-3 of the projection maximum: above the float32 parity
  * bound, so GJP_PATH_AUTO never takes it.
  *
+ * GJP_PATH_AUTO takes the column form of the forward for scans whose
+ * detector rows run along z (det_v parallel to z in every view, slopes
+ * along z below 1/2) on grids of 112 to 1024 voxels along z, a multiple of
+ * 4, with 32-bit offsets, a volume aligned to 4 voxels, more than 2^22 voxels
+ * (16-bit storage: 2^25), enough columns and views to fill the GPU and line
+ * and detector lengths that fill its warps: a block interpolates whole z
+ * lines between the two rows of a plane once for all rays of a detector
+ * column and samples them from shared memory.  It allocates nothing, and its
+ * results agree with GATHER's to float32 rounding.
+ *
  * PAIRS first writes a z-paired copy of the volume, whose element e holds
  * voxels e and e + 1 of the same z line (the upper one zero past the last
  * z), and the row-table march of GATHER then reads both z taps of a row with
@@ -216,7 +226,7 @@ typedef enum {
  * gjp_trim_workspace).  PAIRS returns GJP_ERR_UNSUPPORTED while `stream`
  * is being captured into a CUDA graph and for grids whose element offsets
  * do not fit 32 bits, and GJP_ERR_OOM when the copy cannot be allocated.
- * GJP_PATH_AUTO takes PAIRS for bfloat16 and float16 storage when g has at
+ * Otherwise GJP_PATH_AUTO takes PAIRS for bfloat16 and float16 storage when g has at
  * least 32 views and views x voxels is at least 2^27 (measured faster than
  * GATHER there: half the load instructions, same L1 lines per load; with
  * fewer views the volume is read from DRAM about once and the copy only
@@ -358,9 +368,9 @@ gjp_status gjp_footprint(const gjp_geometry *g, int view, int64_t nx, int64_t ny
  * plug-in that must not touch its host application's allocator.
  *
  * It computes exactly what gjp_forward computes (the same per-view table
- * and the same gather kernels, so the projections are bitwise equal; it
- * always reads the volume itself, never a z-paired copy, whose taps are
- * the same values), but
+ * and the same kernels, so the projections are bitwise equal; it always
+ * reads the volume itself, never a z-paired copy, whose taps are the same
+ * values), but
  * keeps the per-view table in a fixed array of GJP_NOALLOC_MAX_VIEWS entries
  * (144 bytes each, about 144 KiB) that the CUDA runtime places on every GPU
  * that loads this library and keeps there until the process exits.  The
@@ -431,8 +441,9 @@ void gjp_batch_destroy(gjp_batch *b);
 
 /*
  * gjp_batch_forward -- the problems of the batch on `stream`: a problem
- * whose work items fill the GPU's resident blocks 16 times or more runs as
- * its own launch of the gather forward (the kernels of gjp_forward; a
+ * that gjp_forward projects with its column form, or whose work items fill
+ * the GPU's resident blocks 16 times or more, runs as its own launch of the
+ * column form or the gather forward (the kernels of gjp_forward; of the latter a
  * bfloat16 or float16 one where AUTO would take the copy first rewrites its
  * z-paired copy, allocated by gjp_batch_create and kept with the batch), and all
  * other problems share one persistent kernel launch (preceded by a 4-byte

@@ -190,6 +190,7 @@ struct gjp_batch {
     BatchProblem *d_tune = nullptr;      // one-problem queue for the autotuner
     long long *d_tune_begins = nullptr;
     std::vector<char> solo;              // per problem (queue order): its own launch
+    std::vector<char> columns;           // per problem: a solo launch of the forward's column form
     std::vector<void *> solo_pairs;      // per problem: the z-paired copy of a solo 16-bit problem, or null
     int n_queue = 0;                     // problems in the persistent queue
 };
@@ -243,6 +244,10 @@ gjp_status run_batch(const gjp_batch *b, cudaStream_t s)
             if (write_zpairs16(P.vol, dt, n, pairs, s) != cudaSuccess) return GJP_ERR_CUDA;
         }
         const GatherShape sh{P.nu, P.nv, P.n_views, P.tile_u, P.view_group, (P.kind & 8) != 0};
+        if (b->columns[q]) {
+            if (forward_columns(P.vol, dt, P.V, P.table, sh, P.proj, s) != cudaSuccess) return GJP_ERR_CUDA;
+            continue;
+        }
         if (forward_gather_shaped(P.vol, dt, P.V, P.table, sh, (P.kind & 4) != 0, P.proj, pairs, s) != cudaSuccess)
             return GJP_ERR_CUDA;
     }
@@ -283,9 +288,11 @@ gjp_status gjp_batch_create(const gjp_problem *problems, int count, gjp_batch **
     if (!b) return GJP_ERR_OOM;
     std::vector<BatchProblem> host;
     std::vector<int> planes;
+    std::vector<char> columns;
     try {
         host.resize(count);
         planes.resize(count);
+        columns.resize(count);
     } catch (const std::bad_alloc &) {
         delete b;
         return GJP_ERR_OOM;
@@ -325,6 +332,7 @@ gjp_status gjp_batch_create(const gjp_problem *problems, int count, gjp_batch **
         const int tu = valid_tile(q.geometry->tile_u) ? q.geometry->tile_u : 4;
         shape_problem(P, tu, launch_view_group(*q.geometry, n), q.geometry->n_views);
         planes[p] = (int)std::max(n[0], std::max(n[1], n[2]));
+        columns[p] = takes_columns(q.geometry, entry, n, h, q.dtype, q.d_volume) ? 1 : 0;
     }
     // queue order: problems with the longest rays (most planes per item) first
     std::vector<int> order(count);
@@ -334,6 +342,7 @@ gjp_status gjp_batch_create(const gjp_problem *problems, int count, gjp_batch **
     for (int p : order) {
         b->probs.push_back(host[p]);
         b->full_views.push_back(host[p].n_views);
+        b->columns.push_back(columns[p]);
     }
     const size_t pb = sizeof(BatchProblem) * count, bb = sizeof(long long) * (count + 1);
     if (!alloc_gate() || cudaMalloc(&b->d_probs, pb) != cudaSuccess || cudaMalloc(&b->d_begins, bb) != cudaSuccess ||
@@ -359,7 +368,8 @@ gjp_status gjp_batch_create(const gjp_problem *problems, int count, gjp_batch **
         return GJP_ERR_CUDA;
     }
     b->grid = per_sm * sms;
-    // problems that fill the GPU alone run as their own launch; a 16-bit
+    // problems that gjp_forward projects with its column form, and those that
+    // fill the GPU alone, run as their own launch; of the latter a 16-bit
     // one reads a z-paired copy kept with the batch where gjp_forward's AUTO
     // would (pairs_pay), unless it cannot be allocated
     try {
@@ -371,8 +381,9 @@ gjp_status gjp_batch_create(const gjp_problem *problems, int count, gjp_batch **
     }
     for (int q = 0; q < count; ++q) {
         const BatchProblem &P = b->probs[q];
-        if (P.items < (long long)kSoloWaves * b->grid) continue;
+        if (!b->columns[q] && P.items < (long long)kSoloWaves * b->grid) continue;
         b->solo[q] = 1;
+        if (b->columns[q]) continue;
         const int64_t dims[3] = {P.V.n[0], P.V.n[1], P.V.n[2]};
         if ((P.kind & 3) == GJP_F32 || !(P.kind & 4) || !pairs_pay(P.n_views, dims)) continue;
         const size_t bytes = (size_t)P.V.n[0] * P.V.n[1] * P.V.n[2] * sizeof(unsigned);

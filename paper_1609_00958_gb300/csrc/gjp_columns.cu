@@ -38,6 +38,56 @@ constexpr int kColWarps = 4;                 // warps per block: neighbouring pl
 // Host: whether a scan on a grid has the column form, and the per-view
 // records of the column search.
 
+// The smallest driving component over the columns of a view with direction
+// r0 + u ru (|u| <= cu): at an end or where |r_x| = |r_y| or a component
+// vanishes, since max(|r_x|, |r_y|) is convex in u.  `changes` counts the
+// places between the ends where |r_x| = |r_y|, the last one at `change`.
+static double least_lateral(const double r0[3], const double ru[3], double cu, int &changes, double &change)
+{
+    const auto lateral = [&](double u) { return std::max(std::fabs(r0[0] + u * ru[0]), std::fabs(r0[1] + u * ru[1])); };
+    const double cand[4] = {(r0[1] - r0[0]) / (ru[0] - ru[1]), -(r0[0] + r0[1]) / (ru[0] + ru[1]), -r0[0] / ru[0],
+                            -r0[1] / ru[1]};
+    double least = std::min(lateral(-cu), lateral(cu));
+    changes = 0;
+    for (int c = 0; c < 4; ++c)
+        if (cand[c] > -cu && cand[c] < cu) {        // false for nan
+            least = std::min(least, lateral(cand[c]));
+            if (c < 2) {
+                ++changes;
+                change = cand[c];
+            }
+        }
+    return least;
+}
+
+// Ray direction of view k (index units) at the detector's centre, and per column.
+static void view_direction(const gjp_geometry &g, int k, const double h[3], double r0[3], double ru[3])
+{
+    const double cu = 0.5 * (g.nu - 1), cv = 0.5 * (g.nv - 1);
+    for (int a = 0; a < 3; ++a) {
+        ru[a] = g.du[3 * k + a] / h[a];
+        r0[a] = (g.org[3 * k + a] - g.src[3 * k + a]) / h[a] + cu * ru[a] + cv * g.dv[3 * k + a] / h[a];
+    }
+}
+
+// Whether the forward's column form covers a scan: detector rows along z in
+// every view and slopes along z below 1/2.
+bool column_rays(const gjp_geometry &g, const double h[3])
+{
+    if (g.nv > (1 << 15)) return false;
+    for (int k = 0; k < g.n_views; ++k)
+        if (g.dv[3 * k] != 0.0 || g.dv[3 * k + 1] != 0.0) return false;
+    const double cu = 0.5 * (g.nu - 1), cv = 0.5 * (g.nv - 1);
+    for (int k = 0; k < g.n_views; ++k) {
+        double r0[3], ru[3], change;
+        int changes;
+        view_direction(g, k, h, r0, ru);
+        const double rise = std::fabs(r0[2]) + cu * std::fabs(ru[2]) + cv * std::fabs(g.dv[3 * k + 2] / h[2]);
+        if (!(rise < 0.49 * least_lateral(r0, ru, cu, changes, change))) return false;
+    }
+    return true;
+}
+
 // Every view needs det_v parallel to z, rays driven by x or y only (with a
 // margin, so that float32 and float64 agree), one change of driving axis
 // across the detector at most, the whole grid in front of the source, and a
@@ -55,30 +105,13 @@ bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], c
     plan.pitch_max = 0.0;
     const double cu = 0.5 * (g.nu - 1), cv = 0.5 * (g.nv - 1);
     for (int k = 0; k < g.n_views; ++k) {
-        double s[3], r0[3], ru[3];
-        const double pv = g.dv[3 * k + 2] / h[2];
-        for (int a = 0; a < 3; ++a) {
-            s[a] = (g.src[3 * k + a] - o[a]) / h[a];
-            ru[a] = g.du[3 * k + a] / h[a];
-            r0[a] = (g.org[3 * k + a] - g.src[3 * k + a]) / h[a] + cu * ru[a] + (a == 2 ? cv * pv : 0.0);
-        }
-        const auto at = [&](int a, double u) { return r0[a] + u * ru[a]; };
-        const auto lateral = [&](double u) { return std::max(std::fabs(at(0, u)), std::fabs(at(1, u))); };
-        // the smallest driving component: at an end or where |r_x| = |r_y|
-        // or a component vanishes (max(|r_x|, |r_y|) is convex in u)
-        const double cand[4] = {(r0[1] - r0[0]) / (ru[0] - ru[1]), -(r0[0] + r0[1]) / (ru[0] + ru[1]),
-                                -r0[0] / ru[0], -r0[1] / ru[1]};
-        double least = std::min(lateral(-cu), lateral(cu));
+        double s[3], r0[3], ru[3], change = 0.0;
         int changes = 0;
-        double change = 0.0;
-        for (int c = 0; c < 4; ++c)
-            if (cand[c] > -cu && cand[c] < cu) {        // false for nan
-                least = std::min(least, lateral(cand[c]));
-                if (c < 2) {
-                    ++changes;
-                    change = cand[c];
-                }
-            }
+        const double pv = g.dv[3 * k + 2] / h[2];
+        for (int a = 0; a < 3; ++a) s[a] = (g.src[3 * k + a] - o[a]) / h[a];
+        view_direction(g, k, h, r0, ru);
+        const auto at = [&](int a, double u) { return r0[a] + u * ru[a]; };
+        const double least = least_lateral(r0, ru, cu, changes, change);
         if (changes > 1) return false;
         if (!(std::fabs(r0[2]) + cu * std::fabs(ru[2]) + cv * std::fabs(pv) < 0.999 * least)) return false;
         for (int m = 0; m < 2; ++m) {
@@ -124,17 +157,11 @@ bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], c
 // that the driving axis and the transverse position agree with the forward's
 // bit for bit; the z position and its pitch per row follow from the moment's
 // and the direction's dependence on v.
-__global__ void gjp_columns_kernel(const ViewParams *__restrict__ views, VolParams V, int nu, int n_views,
-                                   Column *__restrict__ cols)
+__device__ __forceinline__ Column make_column(const ViewParams &vp, const VolParams &V, float fu)
 {
-    const int u = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
-    if (u >= nu) return;
-    ViewParams vp;
-    load_view(views, k, vp);
     Ray R;
-    setup_ray(vp, V, (float)u - 0.5f * (float)(nu - 1), 0.0f, R);
+    setup_ray(vp, V, fu, 0.0f, R);
     const int m = R.m, a = 1 - m;
-    const float fu = (float)u - 0.5f * (float)(nu - 1);
     const auto lateral = [&](int k) {
         return f2_affine({vp.rh[k], vp.rl[k]}, {vp.rh[3 + k], vp.rl[3 + k]}, {vp.rh[6 + k], vp.rl[6 + k]}, fu, 0.0f);
     };
@@ -156,7 +183,17 @@ __global__ void gjp_columns_kernel(const ViewParams *__restrict__ views, VolPara
     c.Y1 = __float2ll_rn(dg.hi * scale) + __float2ll_rn(dg.lo * scale);
     c.m = m;
     c.pad = 0;
-    cols[(size_t)k * nu + u] = c;
+    return c;
+}
+
+__global__ void gjp_columns_kernel(const ViewParams *__restrict__ views, VolParams V, int nu, int n_views,
+                                   Column *__restrict__ cols)
+{
+    const int u = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    if (u >= nu) return;
+    ViewParams vp;
+    load_view(views, k, vp);
+    cols[(size_t)k * nu + u] = make_column(vp, V, (float)u - 0.5f * (float)(nu - 1));
 }
 
 cudaError_t write_columns(const ViewParams *views, const VolParams &V, const gjp_geometry &g, Column *cols,
@@ -638,6 +675,260 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
     }
     const cudaError_t f = cudaFreeAsync(ws, s);
     return e == cudaSuccess && f == cudaSuccess ? GJP_OK : GJP_ERR_CUDA;
+}
+
+// ---------------------------------------------------------------------------
+// Forward, column form.
+//
+// The forward of one detector column separates the same way: on plane i its
+// rays sample one line of z, W[z] = (1 - d_a) V[ia][z] + d_a V[ia + 1][z].
+// A block owns a column (all its rays, or a part of them): its threads form
+// W for kPhase planes from whole z lines, read in aligned 16-byte words, and
+// leave it in shared memory; then each ray takes its two z taps of W from
+// there.  Against the gather's four unaligned loads per sample (two 128-byte
+// lines each, which bound it) this reads each row of a plane once per column
+// in whole lines, and a sample is one interpolation.  512^3 / 360 views: f32
+// 35.2 -> 31.0 ms, bf16 31.6 -> 29.8 ms.  Shared-memory and L1 wavefronts (78%)
+// and issue (64%, 17.7 instructions per sample and its share of the lines)
+// bound it at 16 warps per SM; 20 or 24 warps cost spills (34.8, 43.0 ms), two planes
+// per step more barriers (37 ms), eight more registers (36.9 ms), and skipping
+// the part of a line that no ray needs more than it saves (36.1 ms).
+
+constexpr int kPhase = 4;            // planes per step
+constexpr int kLineEdge = 4;         // words before (and after) a line in shared memory: zeros at its ends
+
+template <typename T> struct Quad { using type = float4; };
+template <> struct Quad<__nv_bfloat16> { using type = uint2; };
+template <> struct Quad<__half> { using type = uint2; };
+template <typename T> __device__ __forceinline__ float4 widen_quad(typename Quad<T>::type q)
+{
+    if constexpr (std::is_same<T, float>::value) return q;
+    else
+        return make_float4(widen<T>((unsigned short)(q.x & 0xffffu)), widen<T>((unsigned short)(q.x >> 16)),
+                           widen<T>((unsigned short)(q.y & 0xffffu)), widen<T>((unsigned short)(q.y >> 16)));
+}
+
+template <typename T, int RAYS, bool SPL>
+__global__ void __launch_bounds__(256, 2) gjp_forward_columns_kernel(
+    const T *__restrict__ vol, VolParams V, const ViewParams *__restrict__ views, int nu, int nv, int n_vt, int n_views,
+    int view_group, float *__restrict__ proj)
+{
+    using Q = typename Quad<T>::type;
+    extern __shared__ __align__(16) float s_lines[];     // [2][kPhase][kLineEdge + nz + kLineEdge]
+    int tile, view;
+    block_tile_view(n_views, view_group, tile, view);
+    const int nt = blockDim.x, tid = threadIdx.x;
+    const int iu = tile / n_vt, iv0 = (tile % n_vt) * RAYS * nt + tid;   // rays iv0 + j nt
+    const int nz = V.n[2], stride = nz + 2 * kLineEdge;
+
+    Column c;
+    {
+        ViewParams vp;
+        load_view(views, view, vp);
+        c = make_column(vp, V, (float)iu - 0.5f * (float)(nu - 1));
+    }
+    const int m = c.m, nm = m == 0 ? V.n[0] : V.n[1], na = m == 0 ? V.n[1] : V.n[0];
+    const int sm = (int)(m == 0 ? V.s[0] : V.s[1]), sa = (int)(m == 0 ? V.s[1] : V.s[0]);
+    const int ic = (nm - 1) >> 1;
+    int i0, i1, j0, j1;                                   // planes on which the column meets the grid
+    plane_ranges(c.Pa, c.Ga, ic, na, nm, i0, i1, j0, j1);
+    if (V.fov_r2 > 0.0f) {
+        int lo, hi;
+        fov_planes(V, m, ic, c.Pa, c.Ga, 0, 0, lo, hi);   // z plays no part
+        i0 = max(i0, lo);
+        i1 = min(i1, hi);
+    }
+
+    // rays: position on the next plane, increment (|.| < 1/2: it fits 32
+    // fraction bits with its sign), and the planes on which some ray of the
+    // warp meets the z range of the grid, and on which all do
+    long long pb[RAYS];
+    int gb[RAYS], any_lo[RAYS], any_hi[RAYS], all_lo[RAYS], all_hi[RAYS];
+    float2 acc[RAYS], blk[RAYS];
+#pragma unroll
+    for (int j = 0; j < RAYS; ++j) {
+        const long long v2 = 2 * min(iv0 + j * nt, nv - 1) - (nv - 1);   // twice the centred row
+        const long long P = c.Z0 + ((v2 * c.Y0) >> (kPitchBits - 31)), G = c.Z1 + ((v2 * c.Y1) >> (kPitchBits - 31));
+        int z0, z1, k0, k1;
+        plane_ranges(P, G, ic, nz, nm, z0, z1, k0, k1);
+        any_lo[j] = __reduce_min_sync(0xffffffffu, z0 <= z1 ? z0 : INT_MAX);
+        any_hi[j] = __reduce_max_sync(0xffffffffu, z0 <= z1 ? z1 : -1);
+        all_lo[j] = __reduce_max_sync(0xffffffffu, z0);
+        all_hi[j] = __reduce_min_sync(0xffffffffu, z1);
+        pb[j] = pos_at(P, G, i0, ic);
+        gb[j] = (int)G;
+        acc[j] = blk[j] = make_float2(0.0f, 0.0f);
+    }
+    for (int k = tid; k < 2 * kPhase * 2 * kLineEdge; k += nt) {     // the zeros at the lines' ends
+        const int line = k / (2 * kLineEdge), e = k % (2 * kLineEdge);
+        s_lines[line * stride + (e < kLineEdge ? e : nz + e)] = 0.0f;
+    }
+
+    unsigned long long pa = (unsigned long long)pos_at(c.Pa, c.Ga, i0, ic);
+    const bool mine = 4 * tid < nz;
+    int base = i0 * sm + 4 * tid;
+    Q lo[kPhase], hi[kPhase];
+    float da[kPhase];
+    const auto fetch = [&](int i) {                       // rows of planes i .. i + kPhase - 1
+        const bool inside = i >= j0 && i + kPhase - 1 <= min(i1, j1);   // both rows of every plane in the grid
+        if (inside && mine) {
+#pragma unroll
+            for (int t = 0; t < kPhase; ++t) {
+                da[t] = upper_weight<SPL>(frac_of(pa));
+                const int off = base + floor_of(pa) * sa;
+                lo[t] = __ldg(reinterpret_cast<const Q *>(vol + off));
+                hi[t] = __ldg(reinterpret_cast<const Q *>(vol + (off + sa)));
+                pa += (unsigned long long)c.Ga;
+                base += sm;
+            }
+        } else {
+#pragma unroll
+            for (int t = 0; t < kPhase; ++t) {
+                const int ia = floor_of(pa);
+                da[t] = upper_weight<SPL>(frac_of(pa));
+                const bool in = mine && i + t <= i1;
+                const int off = base + ia * sa;
+                lo[t] = in && ia >= 0 ? __ldg(reinterpret_cast<const Q *>(vol + off)) : Q{};
+                hi[t] = in && ia + 1 < na ? __ldg(reinterpret_cast<const Q *>(vol + (off + sa))) : Q{};
+                pa += (unsigned long long)c.Ga;
+                base += sm;
+            }
+        }
+    };
+    // one ray's samples of a phase; CLAMP: outside the z range both taps are a line's end zeros
+    const auto sample = [&](const float *lines, long long &pos, int step, float2 &sum, auto clamp) {
+#pragma unroll
+        for (int t = 0; t < kPhase; t += 2) {
+            const long long p0 = pos, p1 = pos + step;
+            int z0 = floor_of((unsigned long long)p0), z1 = floor_of((unsigned long long)p1);
+            if (decltype(clamp)::value) {
+                z0 = min(max(z0, -2), nz);
+                z1 = min(max(z1, -2), nz);
+            }
+            const float *l0 = lines + t * stride + z0, *l1 = lines + (t + 1) * stride + z1;
+            const float2 lower = make_float2(l0[0], l1[0]), upper = make_float2(l0[1], l1[1]);
+            const float2 d = __ffma2_rn(lower, make_float2(-1.0f, -1.0f), upper);
+            sum = __fadd2_rn(sum, __ffma2_rn(upper_weight2<SPL>((unsigned long long)p0, (unsigned long long)p1), d, lower));
+            pos = p1 + step;
+        }
+    };
+    if (i0 <= i1) fetch(i0);
+    int buf = 0, phases = 0;
+    for (int i = i0; i <= i1; i += kPhase) {
+        float *lines = s_lines + buf * kPhase * stride + kLineEdge;
+        if (mine) {
+#pragma unroll
+            for (int t = 0; t < kPhase; ++t) {
+                const float4 a = widen_quad<T>(lo[t]), b = widen_quad<T>(hi[t]);
+                const float2 m1 = make_float2(-1.0f, -1.0f), w = make_float2(da[t], da[t]);
+                const float2 x = make_float2(a.x, a.y), y = make_float2(a.z, a.w);
+                const float2 p = __ffma2_rn(w, __ffma2_rn(x, m1, make_float2(b.x, b.y)), x);
+                const float2 q = __ffma2_rn(w, __ffma2_rn(y, m1, make_float2(b.z, b.w)), y);
+                *reinterpret_cast<float4 *>(lines + t * stride + 4 * tid) = make_float4(p.x, p.y, q.x, q.y);
+            }
+        }
+        __syncthreads();        // lines complete; every warp is done with the other buffer's last lines
+        if (i + kPhase <= i1) fetch(i + kPhase);
+#pragma unroll
+        for (int j = 0; j < RAYS; ++j) {
+            if (i >= all_lo[j] && i + kPhase - 1 <= all_hi[j])
+                sample(lines, pb[j], gb[j], blk[j], std::false_type{});
+            else if (i <= any_hi[j] && i + kPhase - 1 >= any_lo[j])
+                sample(lines, pb[j], gb[j], blk[j], std::true_type{});
+            else
+                pb[j] += (long long)kPhase * gb[j];
+        }
+        buf ^= 1;
+        if ((++phases % (16 / kPhase)) == 0) {            // 16 planes: join the total
+#pragma unroll
+            for (int j = 0; j < RAYS; ++j) {
+                acc[j] = __fadd2_rn(acc[j], blk[j]);
+                blk[j] = make_float2(0.0f, 0.0f);
+            }
+        }
+    }
+    const float hm = m == 0 ? V.h[0] : V.h[1], ha = m == 0 ? V.h[1] : V.h[0];
+    const float ga = ha * (__ll2float_rn(c.Ga) * 2.3283064365386963e-10f);
+#pragma unroll
+    for (int j = 0; j < RAYS; ++j) {
+        const int iv = iv0 + j * nt;
+        if (iv >= nv) break;
+        const float2 s = __fadd2_rn(acc[j], blk[j]);
+        const float gz = V.h[2] * ((float)gb[j] * 2.3283064365386963e-10f);
+        proj[((size_t)view * nv + iv) * nu + iu] = (s.x + s.y) * sqrtf(hm * hm + ga * ga + gz * gz);
+    }
+}
+
+// Block shape of the forward's column form: `threads` threads with four
+// voxels of a line each (nz / 4 rounded up to warps) and `rays` rays of the
+// column each; `parts` blocks share a column.
+struct ColumnShape {
+    int threads, rays, parts;
+};
+static ColumnShape column_shape(int nv, int nz)
+{
+    ColumnShape c;
+    c.threads = (nz / 4 + 31) / 32 * 32;
+    const int parts = (nv + 6 * c.threads - 1) / (6 * c.threads);
+    c.rays = std::max(4, (nv + parts * c.threads - 1) / (parts * c.threads));
+    c.parts = (nv + c.rays * c.threads - 1) / (c.rays * c.threads);
+    return c;
+}
+
+// Whether the column form is the faster forward.  A thread's plane costs
+// about 1.8 samples for its part of the line plus one per ray, so idle lanes
+// (lines of nz / 4 threads or rays that do not fill the warps) show in
+// `cost`, 1 for full ones.  Measured against the gather (with its deeper
+// loads and paired copies), gather -> columns:
+//   float32: 512^3 / 360 views 35.2 -> 31.0 ms, 8 views 1.15 -> 0.81 ms; 256^3 / 180 views
+//     2.35 -> 1.98 ms; 128^3 / 32 views 87 -> 71 us; 512x512x128 / 60 views 1.93 -> 1.27 ms;
+//     448^3 / 60 views (cost 1.14) 4.76 -> 4.14 ms; 320^3 / 120 views (1.20) 3.02 -> 3.36 ms;
+//     400^3 with 600^2 pixels / 50 views (1.15) 5.35 -> 5.78 ms.
+//   16-bit: 512^3 / 360 views 31.6 -> 29.8 ms, 16 views 2.27 -> 1.43 ms; 1024^3 / 60 views
+//     53.1 -> 43.5 ms; 448^3 / 60 views (1.14) 4.12 -> 4.13 ms.  Grids up to 2^25
+//     voxels keep the z-paired copy.
+// Fewer than 2048 warps leave SMs idle (256^3, f32: one view 34 us for the gather, 56 us for
+// columns; two views 45, 56; four 70, 60).  Float32 grids up to 2^22 voxels keep the gather,
+// with which AUTO agrees bit for bit there.
+bool forward_columns_pay(const int64_t n[3], int nu, int nv, int n_views, gjp_dtype dt, const void *vol)
+{
+    if (n[2] % 4 != 0 || n[2] < 112 || n[2] > 1024 || n_views > 65535 || !fits_int32(n)) return false;
+    if (reinterpret_cast<uintptr_t>(vol) % (dt == GJP_F32 ? 16 : 8) != 0) return false;
+    const ColumnShape c = column_shape(nv, (int)n[2]);
+    if ((double)n_views * nu * c.parts * (c.threads / 32) < 2048.0) return false;
+    const double voxels = (double)n[0] * n[1] * n[2];
+    const double cost = c.parts * c.threads * (1.8 + c.rays) / (1.45 * nv);
+    if (dt == GJP_F32) return voxels > 4194304.0 && (cost <= 1.06 || (cost <= 1.16 && voxels >= 8.5e7));
+    return cost <= 1.06 && voxels > 33554432.0;
+}
+
+template <typename T>
+cudaError_t launch_columns(const T *vol, const VolParams &V, const ViewParams *table, const GatherShape &sh, float *proj,
+                           cudaStream_t s)
+{
+    const ColumnShape c = column_shape(sh.nv, V.n[2]);
+    const dim3 grid((unsigned)(c.parts * sh.nu), (unsigned)sh.n_views);
+    const size_t smem = (size_t)2 * kPhase * (V.n[2] + 2 * kLineEdge) * sizeof(float);
+#define GJP_COLUMNS(R, S)                                                                                          \
+    gjp_forward_columns_kernel<T, R, S><<<grid, c.threads, smem, s>>>(vol, V, table, sh.nu, sh.nv, c.parts, sh.n_views, \
+                                                                      sh.view_group, proj)
+    switch (c.rays) {
+    case 4: if (sh.spl) GJP_COLUMNS(4, true); else GJP_COLUMNS(4, false); break;
+    case 5: if (sh.spl) GJP_COLUMNS(5, true); else GJP_COLUMNS(5, false); break;
+    default: if (sh.spl) GJP_COLUMNS(6, true); else GJP_COLUMNS(6, false); break;
+    }
+#undef GJP_COLUMNS
+    return cudaGetLastError();
+}
+
+cudaError_t forward_columns(const void *vol, gjp_dtype dt, const VolParams &V, const ViewParams *table,
+                            const GatherShape &sh, float *proj, cudaStream_t s)
+{
+    switch (dt) {
+    case GJP_F32: return launch_columns<float>(static_cast<const float *>(vol), V, table, sh, proj, s);
+    case GJP_BF16: return launch_columns<__nv_bfloat16>(static_cast<const __nv_bfloat16 *>(vol), V, table, sh, proj, s);
+    default: return launch_columns<__half>(static_cast<const __half *>(vol), V, table, sh, proj, s);
+    }
 }
 
 }  // namespace gjp_detail

@@ -130,6 +130,7 @@ struct gjp_cache_entry {
     double key[9];
     ViewParams *d_table;
     ColumnForm columns;
+    int column_rays = -1;                 // forward's column form: covers the scan (1), not (0), not yet known (-1)
     int box_rows, box_cols4, box_cols8;   // slab box sizes for this grid (0 = not computed)
     void *tex = nullptr;                  // texture arrays of the texture families (gjp_texture.cu)
 };
@@ -191,6 +192,11 @@ cudaError_t forward_gather_shaped(const void *vol, gjp_dtype dt, const VolParams
 // Whether a 16-bit forward over n_views views of grid n is worth a z-paired
 // copy (the rule AUTO follows; gjp.cu).
 bool pairs_pay(int n_views, const int64_t n[3]);
+// Whether gjp_forward (AUTO), gjp_forward_noalloc and batches project a problem
+// with the column form of the forward (gjp.cu; e: the geometry's entry for
+// the grid, or null).  All three ask here, so that their results are the same.
+bool takes_columns(const gjp_geometry *g, gjp_cache_entry *e, const int64_t n[3], const double h[3], gjp_dtype dt,
+                   const void *vol);
 // Writes the z-paired copy (4 bytes per voxel) of a bfloat16 or float16 volume.
 cudaError_t write_zpairs16(const void *vol, gjp_dtype dt, const int64_t n[3], void *out, cudaStream_t s);
 // Texture families (gjp_texture.cu): forward through the texture unit, and
@@ -243,6 +249,12 @@ bool columns_pay(int nz, double pitch = 1.0);
 bool columns_pay(const ColumnForm &form, int nz);
 gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnForm &form, const gjp_geometry &g,
                            float *vol, cudaStream_t s);
+// The forward's column form: whether it covers a scan, whether it is the
+// faster one for a problem that it covers, and its launch.
+bool column_rays(const gjp_geometry &g, const double h[3]);
+bool forward_columns_pay(const int64_t n[3], int nu, int nv, int n_views, gjp_dtype dt, const void *vol);
+cudaError_t forward_columns(const void *vol, gjp_dtype dt, const VolParams &V, const ViewParams *table,
+                            const GatherShape &sh, float *proj, cudaStream_t s);
 // Stream-ordered workspace from the library's pool (gjp.cu): GJP_ERR_UNSUPPORTED
 // while s is being captured, GJP_ERR_OOM when there is no room.
 gjp_status workspace_alloc(size_t bytes, cudaStream_t s, void **out);
