@@ -1765,17 +1765,17 @@ cudaError_t launch_gather_pf(const T *vol, gjp_dtype dt, const int64_t n[3], con
 //     768^3, 36 x 0.5 deg (14) 11.0 -> 10.6, 36 x 3 deg 15.3 -> 13.5;
 //     1024^3, 32 x 0.5 deg (8) 25.4 -> 23.0, 32 x 3 deg 40.0 -> 32.7;
 //     256^3, 64 views 0.83 -> 0.85, 16 views 0.239 -> 0.232, one 0.061 -> 0.034;
-//     128^3, 16 views 0.0464 -> 0.0448.
+//     128^3, 16 views 0.0464 -> 0.0448; 64^3, 32 views (4096 warps) 0.0222 -> 0.0212.
 //   16-bit, z-paired: 512^3, 360 x 1 deg 31.6 -> 33.0, 48 x 2 deg (8) 4.46 -> 4.58,
 //     48 x 4 deg (4) 4.74 -> 4.73, 48 x 7.5 deg (2) 5.48 -> 5.06; 768^3, 36 x
 //     0.5 deg (14) 10.26 -> 10.25, 36 x 1 deg (7) 11.2 -> 10.8; 1024^3, 32 x 0.5 deg
 //     (8) 22.7 -> 21.0, 60 x 6 deg 61.6 -> 53.0; 256^3 always slower.
 //   16-bit, from the volume: 512^3, 16 views 1.89 -> 1.84, 4 views 0.631 -> 0.573;
 //     256^3, 8 views 0.137 -> 0.136, 16 views 0.243 -> 0.248.
-bool deep_loads(const int n[3], int n_views, int group, bool f32, bool pairs)
+bool deep_loads(const int n[3], int n_views, int group, bool f32, bool pairs, double warps)
 {
     const double voxels = (double)n[0] * n[1] * n[2];
-    if (f32) return n_views <= 16 || (voxels >= 1.0e8 && group < 16);
+    if (f32) return n_views <= 16 || warps <= 8192.0 || (voxels >= 1.0e8 && group < 16);
     if (pairs) return (voxels >= 2.6e8 && group < 16) || (voxels >= 6.7e7 && group <= 3);
     return n_views <= 8 || (voxels >= 6.7e7 && n_views < 32);
 }
