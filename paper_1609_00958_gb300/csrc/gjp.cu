@@ -1795,7 +1795,7 @@ cudaError_t launch_gather_shaped(const T *vol, const VolParams &V, const ViewPar
     const int nu = sh.nu, nv = sh.nv, nvw = sh.n_views, vgp = sh.view_group;
     const size_t rows = (size_t)sh.tile_u * 32 * sizeof(uint2);   // row tables (32-bit offsets only)
     if (i32 && sh.tile_u <= kTileU && !(pairs && std::is_same<T, float>::value) &&
-        deep_loads(V.n, nvw, vgp, std::is_same<T, float>::value, pairs != nullptr)) {
+        deep_loads(V.n, nvw, vgp, std::is_same<T, float>::value, pairs != nullptr, (double)nvw * n_tv * nu)) {
         if constexpr (!std::is_same<T, float>::value) {
             if (pairs) {
                 auto kern = spl ? gjp_forward_deep_kernel<T, true, true> : gjp_forward_deep_kernel<T, false, true>;
@@ -2321,9 +2321,9 @@ gjp_status gjp_adjoint_ex(const float *d_proj, const gjp_geometry *g, int64_t nx
     }
     const bool spl = g->weight == GJP_WEIGHT_SPL;
     if (path == GJP_PATH_SLAB && spl) return GJP_ERR_UNSUPPORTED;   // the slab adjoint implements w_lin only
-    if (path == GJP_PATH_AUTO && columns_pay((int)n[2])) {
+    if (path == GJP_PATH_AUTO && columns_pay(n, g->n_views)) {
         const ColumnForm *form = get_columns(g, *entry, n, h, o, s);
-        if (form && columns_pay(*form, (int)n[2])) {
+        if (form && columns_pay(*form, n, g->n_views)) {
             st = adjoint_columns(d_proj, make_vol(n, h, g->fov), *form, *g, d_volume, s);
             if (st == GJP_OK || st == GJP_ERR_CUDA) return st;
         }

@@ -254,7 +254,9 @@ __global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__
 
 // The line index of a voxel's rays is found in fixed point: 9 integer and 23
 // fraction bits, the entry's position for the voxel at lane 16 of the first
-// 32 plus the lane's and the 32's share.  kBias keeps it positive.
+// 32 plus the lane's share (29 fraction bits, the upper half of a product) and
+// that of whole pairs and halves of 64 voxels.  Weights then are good to 1e-7
+// (rms), with no bias.  kBias keeps the position positive.
 constexpr int kBias = 64;
 __host__ __device__ constexpr int chunk_of(int K2) { return 64 * K2; }
 // Zeros before and after a line's values: a tile whose z range only touches
@@ -272,12 +274,12 @@ struct ColumnTiles {
 
 // What a tile needs of one column on its plane, shared by the lanes.
 struct __align__(16) ColumnEntry {
-    int c, step, inv;                  // search position, its increment per 32 voxels and per voxel (2^-23 rays)
+    int c, inv;                        // search position (2^-23 rays), its increment per 64 voxels (per voxel: 2^-29)
     float pitch;                       // B
     float w1;                          // weight of the upper row
     unsigned base;                     // element of search position 0 in the lines
     int code;                          // row + 1 | rays << 4
-    int pad;
+    int pad[2];
 };
 
 __device__ __forceinline__ float fma_sat(float a, float b, float c)
@@ -302,10 +304,9 @@ __device__ __forceinline__ void column_sums(const float *__restrict__ lines, con
                                             float2 (&q)[K2])
 {
     const float *line = lines + e.base;
-    unsigned pos = (unsigned)(e.c + lane16 * e.inv);
+    unsigned pos = (unsigned)(e.c + __mulhi(lane16 * (1 << 26), e.inv));
+    const unsigned half = (unsigned)(e.inv + 1) >> 1;
     const float B = e.pitch;
-    const float k0 = N == 2 ? 1.0f + B : 2.0f * B, k1 = N == 2 ? 1.0f - 2.0f * B : 3.0f * B - 1.0f;
-    const float k2 = 2.0f - 4.0f * B;
 #pragma unroll
     for (int p = 0; p < K2; ++p) {
         float2 w[3], y[3];
@@ -313,17 +314,22 @@ __device__ __forceinline__ void column_sums(const float *__restrict__ lines, con
         const float *at[2];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-            at[s] = line + (pos >> 23);
-            f[s] = __uint_as_float((pos & 0x7FFFFFu) | 0x3F800000u);        // 1 + fraction
-            pos += (unsigned)e.step;
+            const unsigned x = s ? pos + half : pos;
+            at[s] = line + (x >> 23);
+            f[s] = __uint_as_float((x & 0x7FFFFFu) | 0x3F800000u);          // 1 + fraction
         }
+        pos += (unsigned)e.inv;
+        // what is left of the ray's step to the next ray (exact), in rays
+        const float2 F = make_float2(f[0], f[1]), m1 = make_float2(-1.0f, -1.0f);
+        const float2 left = __ffma2_rn(F, m1, make_float2(2.0f, 2.0f));
         if (N == 2) {
-            w[0] = make_float2(fma_sat(-f[0], B, k0), fma_sat(-f[1], B, k0));
-            w[1] = make_float2(fma_sat(f[0], B, k1), fma_sat(f[1], B, k1));
+            const float2 past = __fadd2_rn(F, m1);
+            w[0] = make_float2(fma_sat(-past.x, B, 1.0f), fma_sat(-past.y, B, 1.0f));
+            w[1] = make_float2(fma_sat(-left.x, B, 1.0f), fma_sat(-left.y, B, 1.0f));
         } else if (N == 3) {
-            w[0] = make_float2(__fmaf_rn(-f[0], B, k0), __fmaf_rn(-f[1], B, k0));
-            w[1] = make_float2(1.0f - fabsf(__fmaf_rn(-f[0], B, k1)), 1.0f - fabsf(__fmaf_rn(-f[1], B, k1)));
-            w[2] = make_float2(fma_sat(f[0], B, k2), fma_sat(f[1], B, k2));
+            w[0] = __fmul2_rn(left, make_float2(B, B));
+            w[1] = make_float2(1.0f - fabsf(__fmaf_rn(left.x, B, B - 1.0f)), 1.0f - fabsf(__fmaf_rn(left.y, B, B - 1.0f)));
+            w[2] = make_float2(fma_sat(-left.x, B, 2.0f - 2.0f * B), fma_sat(-left.y, B, 2.0f - 2.0f * B));
         }
         if (N > 0) {
 #pragma unroll
@@ -339,7 +345,7 @@ __device__ __forceinline__ void column_sums(const float *__restrict__ lines, con
 #pragma unroll
             for (int j = 1; j < N; ++j) q[p] = __ffma2_rn(w[j], y[j], q[p]);
         } else {
-            float2 d = make_float2(__fmaf_rn(-f[0], B, k0) - 1.0f, __fmaf_rn(-f[1], B, k0) - 1.0f);
+            float2 d = make_float2(__fmaf_rn(left.x, B, -1.0f), __fmaf_rn(left.y, B, -1.0f));
             float2 sum = make_float2(0.0f, 0.0f);
             for (int j = 0; j < n; ++j) {
                 const float2 v = shape<SPL>(make_float2(__saturatef(1.0f - fabsf(d.x)), __saturatef(1.0f - fabsf(d.y))));
@@ -450,14 +456,14 @@ __device__ __forceinline__ int column_fill(const VolParams &V, const Column *__r
             const float reach = (float)(chunk_of(K2) - 16) * x;
             ok = ok && ray - (int)(16.0f * x) < nv + 2 && ray + (int)reach + n + 2 >= 0;
             const float rest = __ll2float_rn(z16 - (((long long)ray * bq) >> (kPitchBits - 32))) * inv32;
-            e.c = __float2int_rn((rest * x + rest * x_lo) * 8388608.0f) + (kBias << 23);
-            e.step = __float2int_rn(x * 268435456.0f) + __float2int_rn(x_lo * 268435456.0f);
-            e.inv = __float2int_rn(__fmaf_rn(x, 8388608.0f, x_lo * 8388608.0f));
+            // (+ 1/2: the lane's share is rounded down)
+            e.c = __float2int_rn(__fmaf_rn(rest * x + rest * x_lo, 8388608.0f, 0.5f)) + (kBias << 23);
+            e.inv = __float2int_rn(x * 536870912.0f) + __float2int_rn(x_lo * 536870912.0f);
             e.pitch = b;
             e.w1 = upper_weight<SPL>(frac_of(pa));
             e.base = (unsigned)(((sp.view - line_view0) * nu + u) * nvp + pad + ray - kBias + (n > 2 ? 1 : 0));
             e.code = (row + 1) | n << 4;
-            e.pad = 0;
+            e.pad[0] = e.pad[1] = 0;
         }
     }
     const unsigned mask = __ballot_sync(0xffffffffu, ok);
@@ -622,15 +628,21 @@ int column_pairs(int nz, double pitch)
 
 // Whether the column form is the faster adjoint: short z lines leave most of
 // a chunk's lanes idle (64^3: 37 us against 33 us for the warp-combined
-// scatter; 256^3: 2.64 ms against 4.37 ms), and with rays far apart most
-// voxels that it visits receive nothing.
-bool columns_pay(int nz, double pitch)
+// scatter; 256^3: 2.64 ms against 4.37 ms), with rays far apart most voxels
+// that it visits receive nothing, and its transposed projections and two
+// passes are not repaid by little work (128^3, 4 views: 37 against 34 us;
+// 200x180x256, 2 views: 49 against 67 us; 128^3, 16 views: 67 against 77 us).
+bool columns_pay(const int64_t n[3], int n_views, double pitch)
 {
-    const int k = column_pairs(nz, pitch);
+    if (n[2] > (1 << 15) || (double)n_views * (double)n[0] * (double)n[1] * (double)n[2] < 16777216.0) return false;
+    const int nz = (int)n[2], k = column_pairs(nz, pitch);
     return 33 * (k + 1) * column_chunks(nz, k) <= nz;
 }
 
-bool columns_pay(const ColumnForm &form, int nz) { return form.pitch_max <= 3.0 && columns_pay(nz, form.pitch); }
+bool columns_pay(const ColumnForm &form, const int64_t n[3], int n_views)
+{
+    return form.pitch_max <= 3.0 && columns_pay(n, n_views, form.pitch);
+}
 
 // Adds A^T proj to vol.
 gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnForm &form, const gjp_geometry &g,

@@ -245,8 +245,8 @@ inline int launch_view_group(const gjp_geometry &g, const int64_t n[3])
 bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], const double o[3], ColumnPlan &plan);
 cudaError_t write_columns(const ViewParams *views, const VolParams &V, const gjp_geometry &g, Column *cols,
                           cudaStream_t s);
-bool columns_pay(int nz, double pitch = 1.0);
-bool columns_pay(const ColumnForm &form, int nz);
+bool columns_pay(const int64_t n[3], int n_views, double pitch = 1.0);
+bool columns_pay(const ColumnForm &form, const int64_t n[3], int n_views);
 gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnForm &form, const gjp_geometry &g,
                            float *vol, cudaStream_t s);
 // The forward's column form: whether it covers a scan, whether it is the

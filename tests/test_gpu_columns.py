@@ -1,5 +1,5 @@
 """The column form of the adjoint (scans with detector rows along z, z lines
-of about 100 voxels and more) against the FP64 oracle's transpose: chunk
+of about 100 voxels and more, 2^24 view-voxels) against the FP64 oracle's transpose: chunk
 sizes and remainders along z, ragged strips and planes, ray pitches from a
 quarter of a voxel to several, both row directions, every option that the
 adjoint takes, non-finite values, and the calls that fall back to the
@@ -29,31 +29,31 @@ def _scan(name):
     """(volume grid, scan) of one case."""
     if name.startswith("nz"):                          # 64, 128, 192 and 256 voxel chunks, with remainders
         nz = int(name[2:])
-        vg = VolumeGeometry.centred((21, 26, nz))
-        return vg, synth.circular(5, 30, nz + 9, 150.0, 300.0, 2.1, angles=[0.1, 0.9, 2.2, 3.3, 5.5])
+        vg = VolumeGeometry.centred((109, 122, nz))
+        return vg, synth.circular(14, 61, nz + 9, 600.0, 1200.0, 2.1, angles=0.1 + 0.437 * np.arange(14))
     if name == "many_views":                           # several passes of 32 views, several view groups
-        vg = VolumeGeometry.centred((18, 20, 128))
-        return vg, synth.circular(75, 23, 40, 150.0, 300.0, 2.0, pitch_v=6.0)
+        vg = VolumeGeometry.centred((42, 44, 128))
+        return vg, synth.circular(75, 23, 40, 200.0, 400.0, 2.0, pitch_v=4.5)
     if name == "one_view":
-        vg = VolumeGeometry.centred((17, 19, 131))
-        return vg, synth.circular(1, 37, 131, 150.0, 300.0, 2.0, angles=[0.4])
-    if name in ("pitch_0.3", "pitch_0.5", "pitch_0.8", "pitch_2.7"):
+        vg = VolumeGeometry.centred((361, 353, 132))
+        return vg, synth.circular(1, 137, 131, 700.0, 1400.0, 2.0, angles=[0.4])
+    if name in ("pitch_0.33", "pitch_0.5", "pitch_0.8", "pitch_2.5"):
         p = float(name[6:])
-        vg = VolumeGeometry.centred((19, 22, 128))
-        return vg, synth.circular(4, 29, int(140 / p), 400.0, 800.0, 2.0, pitch_v=2.0 * p,
-                                  angles=[0.3, 1.2, 2.9, 4.4])
+        vg = VolumeGeometry.centred((119, 122, 128))
+        return vg, synth.circular(10, 59, int(140 / p), 600.0, 1200.0, 2.0, pitch_v=2.0 * p,
+                                  angles=0.3 + 0.62 * np.arange(10))
     if name == "short_detector":                       # rays cover part of the z lines only
-        vg = VolumeGeometry.centred((20, 20, 256))
-        return vg, synth.circular(4, 31, 40, 150.0, 300.0, 2.0, det_shift_v=20.0)
+        vg = VolumeGeometry.centred((100, 97, 256))
+        return vg, synth.circular(8, 61, 40, 300.0, 600.0, 2.0, angles=0.1 + 0.77 * np.arange(8), det_shift_v=20.0)
     if name == "rows_along_minus_z":
-        vg = VolumeGeometry.centred((25, 22, 150))
-        cg = synth.cone_angle_geometry(150, 70, 6, 12.0)
+        vg = VolumeGeometry.centred((125, 122, 150))
+        cg = synth.cone_angle_geometry(150, 70, 9, 12.0)
         cg.det_origin = cg.det_origin + (cg.nv - 1) * cg.det_v
         cg.det_v = -cg.det_v
         return vg, cg
     if name == "helix_off_centre":                     # anisotropic voxels, an origin, a source that moves along z
-        vg = VolumeGeometry((27, 31, 141), (0.9, 1.1, 1.3), (-10.0, -19.0, -83.0))
-        cg = synth.circular(9, 33, 150, 160.0, 330.0, 2.1, pitch_v=2.7, det_shift_u=2.3)
+        vg = VolumeGeometry((127, 131, 141), (0.9, 1.1, 1.3), (-55.0, -74.0, -83.0))
+        cg = synth.circular(9, 73, 150, 400.0, 810.0, 2.1, pitch_v=2.7, det_shift_u=2.3)
         dz = np.linspace(-30.0, 30.0, 9)
         cg.src[:, 2] += dz
         cg.det_origin[:, 2] += dz
@@ -61,8 +61,8 @@ def _scan(name):
     raise KeyError(name)
 
 
-CASES = ["nz99", "nz128", "nz133", "nz192", "nz256", "nz300", "nz517", "many_views", "one_view", "pitch_0.3", "pitch_0.5",
-         "pitch_0.8", "pitch_2.7", "short_detector", "rows_along_minus_z", "helix_off_centre"]
+CASES = ["nz99", "nz128", "nz133", "nz192", "nz256", "nz300", "nz517", "many_views", "one_view", "pitch_0.33", "pitch_0.5",
+         "pitch_0.8", "pitch_2.5", "short_detector", "rows_along_minus_z", "helix_off_centre"]
 
 
 def _rows(cg, seed=3):
@@ -90,7 +90,7 @@ def test_column_adjoint_field_of_view(gjp):
     parity tests pin against the oracle)."""
     vg, cg = _scan("helix_off_centre")
     g = gjp.Geometry.from_cone(cg)
-    g.set_fov(12.3)
+    g.set_fov(52.3)
     y = torch.from_numpy(_rows(cg)).cuda()
     ref = gjp.adjoint(y, g, vg.n, vg.h, vg.origin, path="gather")
     back = gjp.adjoint(y, g, vg.n, vg.h, vg.origin)
@@ -113,7 +113,7 @@ def test_column_adjoint_non_finite_values(gjp, value):
     """A non-finite pixel reaches the voxels of its own ray and no others."""
     vg, cg = _scan("nz128")
     y = _rows(cg)
-    y[2, 70, 13] = value
+    y[2, 70, 33] = value
     g = gjp.Geometry.from_cone(cg)
     d = torch.from_numpy(y).cuda()
     ref = gjp.adjoint(d, g, vg.n, vg.h, vg.origin, path="gather")
