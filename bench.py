@@ -34,6 +34,7 @@ from __future__ import annotations
 import argparse
 import hashlib
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -262,8 +263,9 @@ def peaks():
 
 COUNTERS = os.path.join("profiles", "ncu_counters.json")
 # the kernel each step entry runs (ncu kernel-name prefix)
-KERNEL_NAMES = {"forward_f32": "gjp_forward_kernel<float", "forward_bf16": "gjp_forward_kernel<__nv_bfloat16",
-                "forward_f16": "gjp_forward_tld4_kernel<__half", "adjoint_f32": "gjp_adjoint_combine_kernel<int"}
+KERNEL_NAMES = {"forward_f32": "gjp_forward_columns_kernel<float",
+                "forward_bf16": "gjp_forward_columns_kernel<__nv_bfloat16",
+                "forward_f16": "gjp_forward_tld4_kernel<__half", "adjoint_f32": "gjp_adjoint_columns_kernel<4"}
 # ncu metric -> record field
 NCU_FIELDS = {
     "gpu__time_duration.sum": "duration_ns",
@@ -569,14 +571,15 @@ def run_gjp(args):
                    "launch": {"tile_u": geom.launch[0], "view_group": geom.launch[1]},
                    "forward_path": args.forward_path, **({"path16": args.path16} if args.path16 else {}),
                    "tap_source": {"forward_f32": "volume", k16: "z-paired copy, written per call"
-                                  if launches_per_step(args.forward_path, args.path16, vg.n, cg.n_views) > 3 else "volume"},
+                                  if launches_per_step(args.forward_path, args.path16, vg.n, cg.n_views, vg, cg)
+                                  > 2 + adjoint_launches(vg, cg) else "volume"},
                    "step": "forward f32 + forward bf16 + adjoint f32", "samples_per_kernel": samples_per_kernel,
                    "l2": "inputs larger than L2 (no flush)",
                    "parallelism": "one GPU" if world == 1 else
                    f"one scan split by views over {world} GPUs (rank views {scan.start}..{scan.stop - 1}), "
                    "adjoint volumes summed by one all-reduce"},
         "kernels": kernels, "roofline": roofline, "clocks": clocks,
-        "gpu_launches": launches_per_step(args.forward_path, args.path16, vg.n, cg.n_views) * args.steps,
+        "gpu_launches": launches_per_step(args.forward_path, args.path16, vg.n, cg.n_views, vg, cg) * args.steps,
         "e2e": e2e,
     }
     if world == 1 and args.content == "random" and not args.no_phantom and not args.first_views:
@@ -632,18 +635,64 @@ def c1_kernels(gjp, dev, reps: int = 200):
     return out
 
 
-def launches_per_step(path: str, path16, n, n_views: int) -> int:
+def takes_columns(n, nu: int, nv: int, n_views: int, sixteen: bool) -> bool:
+    """Whether AUTO projects with the forward's column form (the library's
+    forward_columns_pay rule; the benchmark's scans have their rows along z)."""
+    nx, ny, nz = (int(v) for v in n)
+    if nz % 4 or not 112 <= nz <= 1024 or nx * ny * nz + 2 * (ny * nz + nz + 1) >= 2147483647:
+        return False
+    threads = -(-nz // 128) * 32
+    rays = max(4, -(-nv // (-(-nv // (6 * threads)) * threads)))
+    parts = -(-nv // (rays * threads))
+    if n_views * nu * parts * (threads // 32) < 2048:
+        return False
+    cost, voxels = parts * threads * (1.8 + rays) / (1.45 * nv), nx * ny * nz
+    if sixteen:
+        return cost <= 1.06 and voxels > 2 ** 25
+    return voxels > 2 ** 22 and (cost <= 1.06 or (cost <= 1.16 and voxels >= 8.5e7))
+
+
+def adjoint_launches(vg, cg) -> int:
+    """Kernel launches of one AUTO adjoint: the transposition and the gather
+    of each 512 MB of transposed projections in the column form (the
+    library's column_pairs, columns_pay and line_pad rules), or one scatter."""
+    nz = int(vg.n[2])
+    pitch = []
+    for k in range(cg.n_views):
+        src = (cg.src[k] - np.array(vg.origin)) / np.array(vg.h)
+        for iu in (0, cg.nu - 1):
+            r = (cg.det_origin[k] + iu * cg.det_u[k] - cg.src[k]) / np.array(vg.h)
+            m = int(abs(r[1]) > abs(r[0]))
+            pitch += [abs((i - src[m]) / r[m] * cg.det_v[k][2] / vg.h[2]) for i in (0, vg.n[m] - 1)]
+    low, best = min(pitch), 1
+    for k, least in ((1, 0.26), (2, 0.26), (3, 0.42), (4, 0.55)):
+        if low > least and -(-nz // (64 * k)) * (k + 1) <= -(-nz // (64 * best)) * (best + 1):
+            best = k
+    if cg.n_views * int(np.prod([int(v) for v in vg.n])) < 2 ** 24 or \
+            33 * (best + 1) * -(-nz // (64 * best)) > nz or max(pitch) > 3.0:
+        return 1
+    pad = math.ceil(64 * best / low) + 16
+    line = (cg.nv + 2 * pad + 31) // 32 * 32
+    views = max(1, min(cg.n_views, (512 << 20) // (4 * line * cg.nu)))
+    return 2 * -(-cg.n_views // views)
+
+
+def launches_per_step(path: str, path16, n, n_views: int, vg=None, cg=None) -> int:
     """The library's kernel launches in one step: forward f32, forward bf16
     and the adjoint, plus the z-paired copy that a "pairs" forward writes
     first (AUTO takes it for 16-bit storage over 32 or more views and 2^27
-    view-voxels; both only where the element offsets fit 32 bits, the
-    library's fits_int32 rule)."""
+    view-voxels that the column form does not take; both only where the
+    element offsets fit 32 bits, the library's fits_int32 rule), and the
+    adjoint's transpositions."""
     nx, ny, nz = (int(v) for v in n)
     fits = nx * ny * nz + 2 * (ny * nz + nz + 1) < 2147483647
     p16 = path16 or path
     pays = n_views >= 32 and n_views * nx * ny * nz >= 2 ** 27      # the library's pairs_pay rule
+    if cg is not None and takes_columns(n, cg.nu, cg.nv, n_views, True):
+        pays = False
     pairs16 = p16 == "pairs" or (p16 == "auto" and pays)
-    return 3 + int(fits and pairs16) + int(fits and path == "pairs")
+    adjoint = adjoint_launches(vg, cg) if cg is not None else 1
+    return 2 + adjoint + int(fits and pairs16) + int(fits and path == "pairs")
 
 
 def phantom_kernels(args, gjp, geom, vg, cg, dev, stream, hbm, peak_kind, k16):
@@ -1196,7 +1245,7 @@ def run_cgls(args):
                  "residual": {str(k): float(f"{hist.residual[k]:.4e}") for k in pick if k < len(hist.residual)},
                  "rmse": {str(k): float(f"{hist.rmse[k]:.4e}") for k in pick if k < len(hist.rmse)}},
         "autograd_step_ms": round(ms_grad, 3),
-        "clocks": clocks, "gpu_launches": 2 * n_iter,
+        "clocks": clocks, "gpu_launches": (1 + adjoint_launches(vg, cg)) * n_iter,
     }), flush=True)
 
 
