@@ -1896,8 +1896,8 @@ gjp_status forward_typed(const void *d_volume, gjp_dtype dt, const int64_t n[3],
         if (!launched) return GJP_ERR_UNSUPPORTED;
         return e == cudaSuccess ? GJP_OK : GJP_ERR_CUDA;
     }
-    // measured on the 512^3 / 512^2 / 360-view workload the gather family is
-    // the fastest, so AUTO takes it; SLAB and PREFETCH run only on request
+    // AUTO takes the column form, pairs or the gather (below); SLAB and
+    // PREFETCH measured slower than the gather and run only on request
     if (path == GJP_PATH_SLAB) {
         BoxSize bs;
         {
@@ -1927,8 +1927,10 @@ gjp_status forward_typed(const void *d_volume, gjp_dtype dt, const int64_t n[3],
     // storage when pairs_pay(), the offsets fit 32 bits and the copy can be
     // allocated (otherwise AUTO reads the volume directly).  Its results are
     // bitwise those of GATHER.  Measured on the 512^3 / 360-view workload it
-    // makes the 16-bit forward 11% faster (copy included) and the float32
+    // makes the 16-bit gather 11% faster (copy included) and the float32
     // one 35% slower (8-byte words: twice the footprint in L1 and L2).
+    // (Scans that the column form covers do not come here: 29.8 ms there
+    // against 31.6 ms with the copy.)
     constexpr bool kPairsAuto = !std::is_same<T, float>::value;
     if (path == GJP_PATH_PAIRS || (path == GJP_PATH_AUTO && kPairsAuto && i32 && pairs_pay(g.n_views, n))) {
         if (!i32) return GJP_ERR_UNSUPPORTED;

@@ -16,9 +16,10 @@
 // memory per voxel, driving axis and view group instead of about two per
 // voxel and view.
 //
-// Measured on 512^3 / 512^2 / 360 views: 38.0 ms, against 68.0 ms for the
+// Measured on 512^3 / 512^2 / 360 views: 38.1 ms, against 68.0 ms for the
 // warp-combined scatter, with a fifth of its error.  Instruction issue bounds
-// it (64% with 16 warps per SM; L1 58%): about 14 instructions for 32 voxels
+// it (65% with 16 warps per SM; L1 56%; 24.8 warp instructions per 32 samples of the
+// forward): about 14 instructions for 32 voxels
 // of one column, 30 per column and warp around them, and 1.3 column voxels
 // per sample of the forward (a column at a tile's edge is visited by both
 // tiles).  8 rows and 256 z fill the registers; fewer rows or a shorter chunk
@@ -700,9 +701,9 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
 // there.  Against the gather's four unaligned loads per sample (two 128-byte
 // lines each, which bound it) this reads each row of a plane once per column
 // in whole lines, and a sample is one interpolation.  512^3 / 360 views: f32
-// 35.2 -> 31.0 ms, bf16 31.6 -> 29.8 ms.  Shared-memory and L1 wavefronts (78%)
-// and issue (64%, 17.7 instructions per sample and its share of the lines)
-// bound it at 16 warps per SM; 20 or 24 warps cost spills (34.8, 43.0 ms), two planes
+// 35.2 -> 31.0 ms, bf16 31.6 -> 29.8 ms.  The L1 data pipe (76%; bf16 66%)
+// and issue (63%; bf16 71%; 20.2 and 21.9 warp instructions per 32 samples, lines
+// included) bound it at 16 warps per SM; 20 or 24 warps cost spills (34.8, 43.0 ms), two planes
 // per step more barriers (37 ms), eight more registers (36.9 ms), and skipping
 // the part of a line that no ray needs more than it saves (36.1 ms).
 
