@@ -30,8 +30,6 @@
 
 namespace gjp_detail {
 
-// Fraction bits of the row pitch B in Column (z positions have 32).
-constexpr int kPitchBits = 40;
 constexpr int kStrip = 8;                    // rows of a tile
 constexpr int kColWarps = 4;                 // warps per block: neighbouring planes of one strip
 
@@ -253,34 +251,12 @@ __global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__
 // ---------------------------------------------------------------------------
 // The gather.
 
-// The line index of a voxel's rays is found in fixed point: 9 integer and 23
-// fraction bits, the entry's position for the voxel at lane 16 of the first
-// 32 plus the lane's share (29 fraction bits, the upper half of a product) and
-// that of whole pairs and halves of 64 voxels.  Weights then are good to 1e-7
-// (rms), with no bias.  kBias keeps the position positive.
-constexpr int kBias = 64;
-__host__ __device__ constexpr int chunk_of(int K2) { return 64 * K2; }
-// Zeros before and after a line's values: a tile whose z range only touches
-// the detector's reads this far beyond it.
-int line_pad(int K2, double pitch) { return (int)std::ceil(chunk_of(K2) / pitch) + 16; }
-int line_length(int nv, int pad) { return (nv + 2 * pad + 31) / 32 * 32; }
-
 int column_chunks(int nz, int K2) { return (nz + chunk_of(K2) - 1) / chunk_of(K2); }
 
 struct ColumnTiles {
     int n_zc, n_strip[2], n_pg[2];     // z chunks; strips of kStrip rows and groups of planes per driving axis
     int first[2];                      // first tile of each driving axis
     int view_lo[2], view_hi[2];        // range of the axis' ColumnViews
-};
-
-// What a tile needs of one column on its plane, shared by the lanes.
-struct __align__(16) ColumnEntry {
-    int c, inv;                        // search position (2^-23 rays), its increment per 64 voxels (per voxel: 2^-29)
-    float pitch;                       // B
-    float w1;                          // weight of the upper row
-    unsigned base;                     // element of search position 0 in the lines
-    int code;                          // row + 1 | rays << 4
-    int pad[2];
 };
 
 __device__ __forceinline__ float fma_sat(float a, float b, float c)
@@ -305,8 +281,8 @@ __device__ __forceinline__ void column_sums(const float *__restrict__ lines, con
                                             float2 (&q)[K2])
 {
     const float *line = lines + e.base;
-    unsigned pos = (unsigned)(e.c + __mulhi(lane16 * (1 << 26), e.inv));
-    const unsigned half = (unsigned)(e.inv + 1) >> 1;
+    unsigned pos = column_position(e, lane16);
+    const unsigned half = column_half(e);
     const float B = e.pitch;
 #pragma unroll
     for (int p = 0; p < K2; ++p) {
@@ -316,7 +292,7 @@ __device__ __forceinline__ void column_sums(const float *__restrict__ lines, con
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const unsigned x = s ? pos + half : pos;
-            at[s] = line + (x >> 23);
+            at[s] = line + column_element(x);
             f[s] = __uint_as_float((x & 0x7FFFFFu) | 0x3F800000u);          // 1 + fraction
         }
         pos += (unsigned)e.inv;
@@ -441,29 +417,9 @@ __device__ __forceinline__ int column_fill(const VolParams &V, const Column *__r
                 fov_planes(V, m, ic, c.Pa, c.Ga, 0, 0, lo, hi);   // z plays no part
                 ok = ok && i >= lo && i <= hi;
             }
-            const float inv32 = 2.3283064365386963e-10f, invp = 9.094947017729282e-13f;   // 2^-32, 2^-kPitchBits
-            const long long bq = llabs(c.Y0 + (long long)di * c.Y1);
-            const float b = __ll2float_rn(bq) * invp;
-            const float b_lo = __ll2float_rn(bq - __float2ll_rn(b * 1099511627776.0f)) * invp;
-            const float x = 1.0f / b;
-            const float x_lo = __fmaf_rn(-b, x, 1.0f) * x - b_lo * x * x;      // 1 / B = x + x_lo
-            const int n = b >= 1.0f ? 2 : (int)ceilf(2.0001f * x);
-            // the tile's 17th voxel (the one below it for N > 2) from the
-            // line's first ray, which is the detector row lowest in z
-            const long long z16 = ((long long)(zc + 16 - (n > 2 ? 1 : 0)) << 32) - c.Z0 - (long long)di * c.Z1 +
-                                  (((long long)(nv - 1) * bq) >> (kPitchBits - 31));
-            const int ray = (int)floorf(__ll2float_rn(z16) * inv32 * x);
-            // some ray of the column near the tile
-            const float reach = (float)(chunk_of(K2) - 16) * x;
-            ok = ok && ray - (int)(16.0f * x) < nv + 2 && ray + (int)reach + n + 2 >= 0;
-            const float rest = __ll2float_rn(z16 - (((long long)ray * bq) >> (kPitchBits - 32))) * inv32;
-            // (+ 1/2: the lane's share is rounded down)
-            e.c = __float2int_rn(__fmaf_rn(rest * x + rest * x_lo, 8388608.0f, 0.5f)) + (kBias << 23);
-            e.inv = __float2int_rn(x * 536870912.0f) + __float2int_rn(x_lo * 536870912.0f);
-            e.pitch = b;
+            ok = column_place<K2>(c, di, zc, nv, pad, ((sp.view - line_view0) * nu + u) * nvp, e) && ok;
             e.w1 = upper_weight<SPL>(frac_of(pa));
-            e.base = (unsigned)(((sp.view - line_view0) * nu + u) * nvp + pad + ray - kBias + (n > 2 ? 1 : 0));
-            e.code = (row + 1) | n << 4;
+            e.code |= row + 1;
             e.pad[0] = e.pad[1] = 0;
         }
     }

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "gjp.h"
+#include "gjp_column_index.h"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -91,15 +92,8 @@ static_assert(4 * kBatch == 16, "the row-table march is written for 4-plane batc
 // limit as GJP_MIN_BLOCKS resident blocks of 4 warps
 constexpr int kMinBlocksMax = (GJP_MIN_BLOCKS * 4 + kMaxTileU - 1) / kMaxTileU;
 
-// Column form (gjp_columns.cu): scans whose detector rows run along z.
-// One detector column of one view: the (x, y) path its rays share and their
-// z positions, in fixed point (32 fraction bits; the pitch kPitchBits).
-struct Column {
-    long long Pa, Ga;       // transverse position on plane ic, increment per plane (as Ray)
-    long long Z0, Z1;       // z of the middle row on plane ic, increment per plane
-    long long Y0, Y1;       // z pitch per detector row on plane ic, increment per plane
-    int m, pad;             // driving axis (0 or 1)
-};
+// Column form (gjp_columns.cu; Column: gjp_column_index.h): scans whose
+// detector rows run along z.
 // One view and driving axis m: source and direction in index units, which
 // give the detector column through a point of plane i, and the columns that
 // m drives.
