@@ -31,6 +31,7 @@
 namespace gjp_detail {
 
 constexpr int kStrip = 8;                    // rows of a tile
+constexpr double kColumnSlack = 0.02;        // columns that the float32 search may be off, and twice what it is
 constexpr int kColWarps = 4;                 // warps per block: neighbouring planes of one strip
 
 // ---------------------------------------------------------------------------
@@ -89,8 +90,9 @@ bool column_rays(const gjp_geometry &g, const double h[3])
 
 // Every view needs det_v parallel to z, rays driven by x or y only (with a
 // margin, so that float32 and float64 agree), one change of driving axis
-// across the detector at most, the whole grid in front of the source, and a
-// row pitch between 0.26 (at most 8 rays within a voxel of one) and 64 voxels.
+// across the detector at most, the whole grid in front of the source, a
+// row pitch between 0.26 (at most 8 rays within a voxel of one) and 64 voxels,
+// and a grid on which the float32 column search is good to half its margin.
 bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], const double o[3], ColumnPlan &plan)
 {
     if (g.n_views > 65535 || (int64_t)g.n_views * g.nu > kMaxColumns || g.nv > (1 << 15) ||
@@ -124,6 +126,7 @@ bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], c
                 continue;
             }
             const double det = r0[m] * ru[a] - r0[a] * ru[m];
+            double least_t = 1e300;
             for (int e = 0; e < 4; ++e) {                 // both are monotone in the plane and in the column
                 const double rm = at(m, (e & 2 ? hi : lo) - cu);
                 const double t = ((e & 1 ? (double)(n[m] - 1) : 0.0) - s[m]) / rm;
@@ -131,18 +134,32 @@ bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], c
                 if (!(t > 0.0) || !(pitch >= 0.26) || !(pitch <= 64.0) || !(spacing >= 0.05)) return false;
                 plan.pitch = std::min(plan.pitch, pitch);
                 plan.pitch_max = std::max(plan.pitch_max, pitch);
+                least_t = std::min(least_t, t);
             }
+            // The column through a point (x, y) of (axis m, axis a): iu - cu =
+            // num / den with num = y r0_m - x r0_a - (s_a r0_m - s_m r0_a),
+            // den = x ru_a - y ru_m - (s_m ru_a - s_a ru_m), s the source.
+            // These moments are formed here in float64, so that a distant
+            // source costs no digits; den is made positive in front of it.
+            const double q = std::copysign(1.0 / (std::fabs(ru[m]) + std::fabs(ru[a])), det);
+            const double num[3] = {q * r0[m], q * r0[a], q * (s[a] * r0[m] - s[m] * r0[a])};
+            const double den[3] = {q * ru[a], q * ru[m], q * (s[m] * ru[a] - s[a] * ru[m])};
+            // float32 error of iu: five roundings of each sum's largest partial
+            // sum (coefficients, products, sums), relative to den = t |q det|
+            const double mx = (double)n[m], my = (double)n[a] + kStrip, eps = 5.9604644775390625e-08;   // 2^-24
+            const double err_num = 5.0 * eps * (my * std::fabs(num[0]) + mx * std::fabs(num[1]) + std::fabs(num[2]));
+            const double err_den = 5.0 * eps * (mx * std::fabs(den[0]) + my * std::fabs(den[1]) + std::fabs(den[2]));
+            const double err = (err_num + (cu + 2.0) * err_den) / (least_t * std::fabs(q * det)) + 8.0 * eps * (cu + 2.0);
+            if (!(err <= 0.5 * kColumnSlack)) return false;
             ColumnView v;
-            v.s_m = (float)s[m];
-            v.s_a = (float)s[a];
-            v.r0_m = (float)r0[m];
-            v.ru_m = (float)ru[m];
-            v.r0_a = (float)r0[a];
-            v.ru_a = (float)ru[a];
+            for (int j = 0; j < 3; ++j) {
+                v.num[j] = (float)num[j];
+                v.den[j] = (float)den[j];
+            }
             v.u_lo = lo;
             v.u_hi = hi;
             v.view = k;
-            v.pad = 0;
+            v.rising = at(m, lo - cu) * det > 0.0 ? 1 : -1;
             plan.views[m].push_back(v);
         }
     }
@@ -356,19 +373,16 @@ __device__ __forceinline__ int column_spans(const ColumnView *__restrict__ cview
     int cnt = 0, u_lo = 0, view = 0;
     if (vb + lane < view_hi) {
         const ColumnView cv = cviews[vb + lane];
-        const float cu = 0.5f * (float)(nu - 1);
-        const float dm = (float)i - cv.s_m;
-        const float e0 = (float)(a0 - 1) - cv.s_a, e1 = (float)(a0 + kStrip) - cv.s_a;
-        const float n0 = dm * cv.ru_a - e0 * cv.ru_m, n1 = dm * cv.ru_a - e1 * cv.ru_m;
-        const float det = cv.r0_m * cv.ru_a - cv.r0_a * cv.ru_m;
-        // in front of the source, n / det is positive; iu grows with the
-        // row as dm det does, without bound where n goes to zero
-        const bool f0 = n0 * det > 0.0f, f1 = n1 * det > 0.0f;
-        const float far = dm * det > 0.0f ? 1.0e9f : -1.0e9f;
-        const float u0 = f0 ? __fdividef(e0 * cv.r0_m - dm * cv.r0_a, n0) + cu : -far;
-        const float u1 = f1 ? __fdividef(e1 * cv.r0_m - dm * cv.r0_a, n1) + cu : far;
-        u_lo = max(cv.u_lo, (int)floorf(fmaxf(fminf(u0, u1) - 0.02f, -1.0f)));
-        const int u_hi = min(cv.u_hi, (int)ceilf(fminf(fmaxf(u0, u1) + 0.02f, 1.0e9f)));
+        const float cu = 0.5f * (float)(nu - 1), x = (float)i, y0 = (float)(a0 - 1), y1 = (float)(a0 + kStrip);
+        const float n0 = x * cv.den[0] - y0 * cv.den[1] - cv.den[2], n1 = x * cv.den[0] - y1 * cv.den[1] - cv.den[2];
+        // in front of the source, den is positive; iu grows or falls with the
+        // row throughout, without bound where den goes to zero
+        const bool f0 = n0 > 0.0f, f1 = n1 > 0.0f;
+        const float far = cv.rising > 0 ? 1.0e9f : -1.0e9f;
+        const float u0 = f0 ? __fdividef(y0 * cv.num[0] - x * cv.num[1] - cv.num[2], n0) + cu : -far;
+        const float u1 = f1 ? __fdividef(y1 * cv.num[0] - x * cv.num[1] - cv.num[2], n1) + cu : far;
+        u_lo = max(cv.u_lo, (int)floorf(fmaxf(fminf(u0, u1) - (float)kColumnSlack, -1.0f)));
+        const int u_hi = min(cv.u_hi, (int)ceilf(fminf(fmaxf(u0, u1) + (float)kColumnSlack, 1.0e9f)));
         cnt = f0 || f1 ? max(0, u_hi - u_lo + 1) : 0;
         view = cv.view;
     }

@@ -94,13 +94,13 @@ constexpr int kMinBlocksMax = (GJP_MIN_BLOCKS * 4 + kMaxTileU - 1) / kMaxTileU;
 
 // Column form (gjp_columns.cu; Column: gjp_column_index.h): scans whose
 // detector rows run along z.
-// One view and driving axis m: source and direction in index units, which
-// give the detector column through a point of plane i, and the columns that
-// m drives.
+// One view and driving axis m: the columns that m drives, and the detector
+// column through a point (x, y) of (axis m, the other lateral axis) in index
+// units, (num0 y - num1 x - num2) / (den0 x - den1 y - den2) + (nu - 1) / 2.
 struct ColumnView {
-    float s_m, s_a, r0_m, ru_m, r0_a, ru_a;
+    float num[3], den[3];
     int u_lo, u_hi;
-    int view, pad;
+    int view, rising;                     // rising: +1 where the column grows with y, -1 where it falls
 };
 constexpr int kMaxColumns = 1 << 22;
 // Host: the views that each driving axis has columns of, and the least and
