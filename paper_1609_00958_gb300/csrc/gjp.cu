@@ -1186,13 +1186,17 @@ __global__ void __launch_bounds__(kMaxThreads) gjp_adjoint_combine_kernel(
     uint2 *rows = row_table(threadIdx.y);
     if (!uniform) {
         // rays one after another along z on the centre plane, a third of a
-        // voxel to 1.7 voxels apart, and less than half a voxel apart across
-        // (z lines shorter than 4 voxels: a row's end could pass for the
-        // next row's start)
+        // voxel to 1.7 voxels apart, and less than half a voxel apart across.
+        // On no plane may a row's end pass for the next row's start: lower
+        // taps then lie less than nb - 1 voxels apart along z, which their
+        // rays' distance on the end planes (it is affine in i) shows.
         const long long one = 1LL << 32;
         const long long za = __shfl_down_sync(full, R.Pa, 1) - R.Pa, zb = __shfl_down_sync(full, R.Pb, 1) - R.Pb;
+        const long long gb = __shfl_down_sync(full, R.Gb, 1) - R.Gb;
+        const long long most = (long long)(R.nb - 2) * one, z0 = pos_at(zb, gb, 0, R.ic), z1 = pos_at(zb, gb, R.nm - 1, R.ic);
+        const bool apart = max(z0, z1) <= most && min(z0, z1) >= -most;
         const bool last = lane == 31;
-        const bool row = R.m == m0 && m0 != 2 && R.nb >= 4 && (last || (2 * za < one && -2 * za < one));
+        const bool row = R.m == m0 && m0 != 2 && R.nb >= 4 && (last || (apart && 2 * za < one && -2 * za < one));
         const bool up = __all_sync(full, row && (last || (3 * zb > one && 10 * zb < 17 * one)));
         const bool down = __all_sync(full, row && (last || (-3 * zb > one && -10 * zb < 17 * one)));
         if (up) skew_march<Index, SPL, CLIP, true>(R, ys, vol);
