@@ -336,9 +336,10 @@ gjp_status gjp_adjoint(const float *d_proj, const gjp_geometry *g, int64_t nx, i
  * pass it, and is added to memory once per driving axis and group of views.
  * It reads a transposed copy of the projections, allocated on `stream` from
  * the library's pool (up to 512 MB at a time, released on `stream`; see
- * gjp_trim_workspace), and per-column records (64 bytes per view and
- * detector column) that its first call for a geometry and grid builds and
- * the geometry keeps.  While `stream` is being captured, or when either
+ * gjp_trim_workspace), and per-column records (56 bytes per view and
+ * detector column) that its first call for a geometry and grid writes on
+ * `stream`, without waiting for it, and the geometry keeps until it is
+ * destroyed.  While `stream` is being captured, or when either
  * cannot be allocated, AUTO takes COMBINE.  GJP_PATH_PREFETCH is not an adjoint family
  * (GJP_ERR_INVALID_ARG).  Results agree to float32 rounding; none is
  * bitwise deterministic.

@@ -236,7 +236,9 @@ gjp_status get_table(const gjp_geometry *gc, const int64_t n[3], const double h[
 
 // The column form of (g, grid) on the entry's device (gjp_columns.cu), built
 // on first use; null when the scan has none, when s is being captured or
-// when there is no room for it.
+// when there is no room for it.  The records are written on s, and nothing
+// waits for them here: whoever reads them waits for form->ready on its own
+// stream.
 const ColumnForm *get_columns(const gjp_geometry *gc, gjp_cache_entry &e, const int64_t n[3], const double h[3],
                               const double o[3], cudaStream_t s)
 {
@@ -268,16 +270,19 @@ const ColumnForm *get_columns(const gjp_geometry *gc, gjp_cache_entry &e, const 
             return nullptr;
         }
         Column *cols = reinterpret_cast<Column *>(d + vbytes);
-        // complete before this returns: any stream may read them from here on
-        if (cudaMemcpy(d, views.data(), sizeof(ColumnView) * views.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaEvent_t ready = nullptr;
+        if (cudaEventCreateWithFlags(&ready, cudaEventDisableTiming) != cudaSuccess ||
+            cudaMemcpyAsync(d, views.data(), sizeof(ColumnView) * views.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
             write_columns(e.d_table, make_vol(n, h, 0.0), *g, cols, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
-            cudaFree(d);
+            cudaEventRecord(ready, s) != cudaSuccess) {
+            if (ready) cudaEventDestroy(ready);
+            cudaFree(d);                          // waits for what is queued
             cudaGetLastError();
             return nullptr;
         }
         f.d_views = reinterpret_cast<ColumnView *>(d);
         f.d_cols = cols;
+        f.ready = ready;
         f.pitch = plan.pitch;
         f.pitch_max = plan.pitch_max;
         f.state = ColumnForm::kReady;
@@ -2129,6 +2134,7 @@ void gjp_geometry_destroy(gjp_geometry *g)
             cudaSetDevice(e.device);
             if (e.d_table) cudaFree(e.d_table);
             cudaFree(const_cast<ColumnView *>(e.columns.d_views));
+            if (e.columns.ready) cudaEventDestroy(e.columns.ready);
             free_texture_cache(e);
         }
         if (have_dev) cudaSetDevice(cur);

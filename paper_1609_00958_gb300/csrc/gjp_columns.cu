@@ -637,7 +637,8 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
     j.pad = pad;
     j.vol = vol;
     j.s = s;
-    cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(unsigned), s);
+    cudaError_t e = cudaStreamWaitEvent(s, form.ready, 0);       // the records, written on another stream perhaps
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, sizeof(unsigned), s);
     for (int v0 = 0; v0 < g.n_views && e == cudaSuccess; v0 += most) {
         j.view0 = v0;
         j.n_views = std::min(most, g.n_views - v0);

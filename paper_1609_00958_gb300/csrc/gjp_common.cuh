@@ -115,6 +115,7 @@ struct ColumnForm {
     State state = kUnknown;
     const ColumnView *d_views = nullptr;      // axis 0's, then axis 1's
     Column *d_cols = nullptr;                 // [view][iu]
+    cudaEvent_t ready = nullptr;              // both are written
     std::vector<int> view_ids[2];
     double pitch = 0.0, pitch_max = 0.0;
 };
