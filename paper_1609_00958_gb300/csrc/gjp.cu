@@ -234,6 +234,14 @@ gjp_status get_table(const gjp_geometry *gc, const int64_t n[3], const double h[
     return GJP_OK;
 }
 
+// Within its scope, this thread's allocations do not disturb a graph capture
+// of another thread.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The column form of (g, grid) on the entry's device (gjp_columns.cu), built
 // on first use; null when the scan has none, when s is being captured or
 // when there is no room for it.  The records are written on s, and nothing
@@ -2334,6 +2342,7 @@ gjp_status gjp_adjoint_ex(const float *d_proj, const gjp_geometry *g, int64_t nx
     const bool spl = g->weight == GJP_WEIGHT_SPL;
     if (path == GJP_PATH_SLAB && spl) return GJP_ERR_UNSUPPORTED;   // the slab adjoint implements w_lin only
     if (path == GJP_PATH_AUTO && columns_pay(n, g->n_views)) {
+        const RelaxedCapture relaxed;
         const ColumnForm *form = get_columns(g, *entry, n, h, o, s);
         if (form && columns_pay(*form, n, g->n_views)) {
             st = adjoint_columns(d_proj, make_vol(n, h, g->fov), *form, *g, d_volume, s);

@@ -1,6 +1,8 @@
 """The first column-form adjoint of a geometry, which builds the geometry's
 column records: it waits for no stream, and other streams read the records
-only once they are written."""
+only once they are written.  No call disturbs another thread's graph capture."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -50,3 +52,34 @@ def test_first_call_waits_for_no_stream(gjp):
     torch.cuda.synchronize()
     gjp.stream_status()
     assert _same(outs[0], ref) and _same(outs[1], ref)
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_call_during_another_threads_capture(gjp, warm):
+    vg, g, y, ref = _case(gjp)
+    if warm:
+        gjp.adjoint(y, g, vg.n, vg.h)
+    out = torch.full(vg.n, 3.0, device="cuda")
+    captured = torch.zeros(1000, device="cuda")
+    errors = []
+
+    def work(stream):
+        try:
+            with torch.cuda.stream(stream):
+                gjp.adjoint(y, g, vg.n, vg.h, out=out)
+        except Exception as e:                           # reported by the test's thread
+            errors.append(e)
+
+    worker = threading.Thread(target=work, args=(torch.cuda.Stream(),))
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        captured += 1.0
+        worker.start()
+        worker.join()
+        captured += 1.0
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not errors
+    assert float(captured[0]) == 2.0
+    assert _same(out, ref)
