@@ -2304,7 +2304,7 @@ gjp_status gjp_stream_status(void *stream)
 {
     if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return GJP_ERR_CUDA;
     if (GJP_CHECK_TAPS) {
-        const unsigned taps = take_tap_faults() | batch_tap_faults() | texture_tap_faults();
+        const unsigned taps = take_tap_faults() | batch_tap_faults() | texture_tap_faults() | columns_tap_faults();
         if (taps) return GJP_ERR_INTERNAL;
     }
     unsigned flag = 0;

@@ -46,7 +46,7 @@ struct alignas(16) ColumnEntry {
     float w1;                          // weight of the upper row
     int base;                          // element of search position 0 in the lines
     int code;                          // row + 1 | rays << 4
-    int pad[2];
+    int line, length;                  // the line's first element and its length (debug build)
 };
 
 GJP_HD int column_round(float x)

@@ -289,6 +289,30 @@ template <bool SPL> __device__ __forceinline__ float2 shape(float2 e)
     return SPL ? __fmul2_rn(__fmul2_rn(e, e), __ffma2_rn(e, make_float2(-2.0f, -2.0f), make_float2(3.0f, 3.0f))) : e;
 }
 
+// Debug build (GJP_CHECK_TAPS): where a lane loads `n` elements of entry e's
+// line from; loads that would leave the line are recorded and read its first
+// elements instead (a line is longer than any n).  The element itself, and
+// free, in the production build.
+__device__ __forceinline__ int checked_element(const ColumnEntry &e, unsigned position, int n)
+{
+    const int k = column_element(position);
+    if (!GJP_CHECK_TAPS) return k;
+    const int in_line = e.base + k - e.line;
+    const bool ok = in_line >= 0 && in_line + n <= e.length;
+    if (!ok) atomicOr(&g_gjp_tap_fault, 1u);
+    return ok ? k : e.line - e.base;
+}
+
+// The same for the taps z0 and z0 + 1 of a forward line of nz voxels with its
+// edges.
+__device__ __forceinline__ int checked_line_tap(int z0, int nz, int edge)
+{
+    if (!GJP_CHECK_TAPS) return z0;
+    const bool ok = z0 >= -edge && z0 + 1 < nz + edge;
+    if (!ok) atomicOr(&g_gjp_tap_fault, 1u);
+    return ok ? z0 : 0;
+}
+
 // Q of one column at the lane's 2 K2 voxels (z = lane + 32 k).  N = 2
 // (B >= 1): the rays on either side of z; N = 3 (B >= 2/3): the first three
 // above z - 1; N = 0: the first n above z - 1.  CAREFUL keeps a ray out of
@@ -309,7 +333,7 @@ __device__ __forceinline__ void column_sums(const float *__restrict__ lines, con
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const unsigned x = s ? pos + half : pos;
-            at[s] = line + column_element(x);
+            at[s] = line + checked_element(e, x, N > 0 ? N : n);
             f[s] = __uint_as_float((x & 0x7FFFFFu) | 0x3F800000u);          // 1 + fraction
         }
         pos += (unsigned)e.inv;
@@ -434,7 +458,8 @@ __device__ __forceinline__ int column_fill(const VolParams &V, const Column *__r
             ok = column_place<K2>(c, di, zc, nv, pad, ((sp.view - line_view0) * nu + u) * nvp, e) && ok;
             e.w1 = upper_weight<SPL>(frac_of(pa));
             e.code |= row + 1;
-            e.pad[0] = e.pad[1] = 0;
+            e.line = GJP_CHECK_TAPS ? ((sp.view - line_view0) * nu + u) * nvp : 0;
+            e.length = GJP_CHECK_TAPS ? nvp : 0;
         }
     }
     const unsigned mask = __ballot_sync(0xffffffffu, ok);
@@ -661,6 +686,8 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
     return e == cudaSuccess && f == cudaSuccess ? GJP_OK : GJP_ERR_CUDA;
 }
 
+unsigned columns_tap_faults() { return take_tap_faults(); }
+
 // ---------------------------------------------------------------------------
 // Forward, column form.
 //
@@ -760,8 +787,9 @@ __global__ void __launch_bounds__(256, 2) gjp_forward_columns_kernel(
             for (int t = 0; t < kPhase; ++t) {
                 da[t] = upper_weight<SPL>(frac_of(pa));
                 const int off = base + floor_of(pa) * sa;
-                lo[t] = __ldg(reinterpret_cast<const Q *>(vol + off));
-                hi[t] = __ldg(reinterpret_cast<const Q *>(vol + (off + sa)));
+                const bool ok = taps_in_grid(i + t, floor_of(pa), 4 * tid + 2, nm, na, nz);   // debug build only
+                lo[t] = ok ? __ldg(reinterpret_cast<const Q *>(vol + off)) : Q{};
+                hi[t] = ok ? __ldg(reinterpret_cast<const Q *>(vol + (off + sa))) : Q{};
                 pa += (unsigned long long)c.Ga;
                 base += sm;
             }
@@ -789,6 +817,8 @@ __global__ void __launch_bounds__(256, 2) gjp_forward_columns_kernel(
                 z0 = min(max(z0, -2), nz);
                 z1 = min(max(z1, -2), nz);
             }
+            z0 = checked_line_tap(z0, nz, kLineEdge);
+            z1 = checked_line_tap(z1, nz, kLineEdge);
             const float *l0 = lines + t * stride + z0, *l1 = lines + (t + 1) * stride + z1;
             const float2 lower = make_float2(l0[0], l1[0]), upper = make_float2(l0[1], l1[1]);
             const float2 d = __ffma2_rn(lower, make_float2(-1.0f, -1.0f), upper);

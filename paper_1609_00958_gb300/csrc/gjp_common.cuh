@@ -257,6 +257,7 @@ gjp_status workspace_alloc(size_t bytes, cudaStream_t s, void **out);
 // (debug build; 0 otherwise), read and cleared.
 unsigned batch_tap_faults();
 unsigned texture_tap_faults();
+unsigned columns_tap_faults();
 
 // ---------------------------------------------------------------------------
 // Device side: double-float helpers (error-free transformations with FMA).
