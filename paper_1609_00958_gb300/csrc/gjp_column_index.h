@@ -69,10 +69,11 @@ GJP_HD int column_mulhi(int a, int b)
 
 // Search position, pitch, ray count and base of column c, di planes from the
 // centre plane, for the chunk of chunk_of(K2) voxels from zc on; `line` is
-// the first element of the column's line.  False when no ray of the column
+// the first element of the column's line, and only its rows first .. end - 1
+// (counted upwards in z) hold anything but zeros.  False when none of these
 // comes near the chunk.
 template <int K2>
-GJP_HD bool column_place(const Column &c, int di, int zc, int nv, int pad, int line, ColumnEntry &e)
+GJP_HD bool column_place(const Column &c, int di, int zc, int nv, int pad, int line, int first, int end, ColumnEntry &e)
 {
     const float inv32 = 2.3283064365386963e-10f, invp = 9.094947017729282e-13f;   // 2^-32, 2^-kPitchBits
     const long long bs = c.Y0 + (long long)di * c.Y1;
@@ -87,9 +88,9 @@ GJP_HD bool column_place(const Column &c, int di, int zc, int nv, int pad, int l
     const long long z16 = ((long long)(zc + 16 - (n > 2 ? 1 : 0)) << 32) - c.Z0 - (long long)di * c.Z1 +
                           (((long long)(nv - 1) * bq) >> (kPitchBits - 31));
     const int ray = (int)floorf((float)z16 * inv32 * x);
-    // some ray of the column near the tile
+    // some such ray of the column near the tile
     const float reach = (float)(chunk_of(K2) - 16) * x;
-    const bool near = ray - (int)(16.0f * x) < nv + 2 && ray + (int)reach + n + 2 >= 0;
+    const bool near = ray - (int)(16.0f * x) < end + 2 && ray + (int)reach + n + 2 >= first;
     const float rest = (float)(z16 - (((long long)ray * bq) >> (kPitchBits - 32))) * inv32;
     // (+ 1/2: the lane's share is rounded down)
     e.c = column_round(fmaf(rest * x + rest * x_lo, 8388608.0f, 0.5f)) + (kBias << 23);

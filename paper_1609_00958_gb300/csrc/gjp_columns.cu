@@ -223,18 +223,40 @@ cudaError_t write_columns(const ViewParams *views, const VolParams &V, const gjp
 // ---------------------------------------------------------------------------
 // The projections, times their plane step, with the detector rows contiguous
 // and ascending in z: line (view, iu) holds y step at pad + row, zeros
-// elsewhere.  Sets
-// *flag when a value is not finite.
+// elsewhere.  Sets head[0] when a value is not finite, and in line_ranges(head)
+// each line's extent of values other than zero, from both ends, so that the
+// gather passes over the rest, as the scatter does over rays of zeros.  512^3
+// / 60 views, without -> with the ranges: zeros 6.40 -> 0.80 ms (the scatter
+// 0.59), one column in 16 6.43 -> 1.14 (1.70), a trace of 32^2 pixels 6.40 ->
+// 1.20 (0.70), dense projections 6.43 -> 6.32 (12.9): the 32-row tiles outside
+// the detector, more than half of them, now only store zeros.
 constexpr int kTrRows = 8;
+
+// Head of the workspace: a flag word, and from byte 256 on one pair per line.
+constexpr size_t kHeadBytes = 256;
+struct LineRange {
+    unsigned from_end, end;            // line length - first such element, last one + 1; zeros: none
+};
+template <typename W> __host__ __device__ __forceinline__ auto line_ranges(W *head)
+{
+    using R = std::conditional_t<std::is_const<W>::value, const LineRange, LineRange>;
+    return reinterpret_cast<R *>(head + kHeadBytes / sizeof(W));
+}
 
 __global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__restrict__ proj, VolParams V,
                                                                   const Column *__restrict__ cols, int nu, int nv,
                                                                   int nvp, int pad, int view0, float *__restrict__ lines,
-                                                                  unsigned *__restrict__ flag)
+                                                                  unsigned *__restrict__ head)
 {
     __shared__ float tile[32][33];
     const int u0 = blockIdx.x * 32, p0 = blockIdx.y * 32;            // p: position in the line
     const int view = view0 + blockIdx.z;
+    if (p0 + 32 <= pad || p0 >= pad + nv) {                          // zeros around the values: more than half of a line
+#pragma unroll
+        for (int k = threadIdx.y; k < 32; k += kTrRows)
+            if (u0 + k < nu) lines[((size_t)blockIdx.z * nu + u0 + k) * nvp + p0 + threadIdx.x] = 0.0f;
+        return;
+    }
     const bool down = cols[(size_t)view * nu].Y0 < 0;                // rows descend in z: reversed lines
     const float *src = proj + (size_t)view * nv * nu;
 #pragma unroll
@@ -250,7 +272,7 @@ __global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__
 #pragma unroll
     for (int k = threadIdx.y; k < 32; k += kTrRows) {
         const int u = u0 + k, p = p0 + threadIdx.x;
-        if (u >= nu || p >= nvp) continue;
+        if (u >= nu) continue;                                       // the whole warp (and p < nvp: a multiple of 32)
         const Column *c = cols + (size_t)view * nu + u;
         const int m = c->m;
         const float hm = m == 0 ? V.h[0] : V.h[1], ha = m == 0 ? V.h[1] : V.h[0];
@@ -260,9 +282,16 @@ __global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__
         const float gb = V.h[2] * __fmaf_rn(v, __ll2float_rn(c->Y1) * vs, __ll2float_rn(c->Z1) * inv);
         const float y = tile[threadIdx.x][k] * sqrtf(hm * hm + ga * ga + gb * gb);
         bad = bad || !(fabsf(y) <= 3.402823466e38f);
-        lines[((size_t)blockIdx.z * nu + u) * nvp + p] = y;
+        const size_t line = (size_t)blockIdx.z * nu + u;
+        lines[line * nvp + p] = y;
+        const unsigned some = __ballot_sync(0xffffffffu, y != 0.0f);
+        if (some && threadIdx.x == 0) {
+            LineRange *r = line_ranges(head) + line;
+            atomicMax(&r->from_end, (unsigned)(nvp - (p0 + __ffs(some) - 1)));
+            atomicMax(&r->end, (unsigned)(p0 + 32 - __clz(some)));
+        }
     }
-    if (bad) atomicOr(flag, 1u);
+    if (bad) atomicOr(head, 1u);
 }
 
 // ---------------------------------------------------------------------------
@@ -429,7 +458,8 @@ __device__ __forceinline__ int column_spans(const ColumnView *__restrict__ cview
 template <int K2, bool SPL>
 __device__ __forceinline__ int column_fill(const VolParams &V, const Column *__restrict__ cols, int nu, int nv, int nvp,
                                            int pad, int line_view0, int m, int i, int a0, int zc,
-                                           const ColumnSpan *__restrict__ spans, int start, bool any, int q0, int total,
+                                           const LineRange *__restrict__ ranges, const ColumnSpan *__restrict__ spans,
+                                           int start, bool any, int q0, int total,
                                            ColumnEntry *__restrict__ tab)
 {
     const unsigned full = 0xffffffffu;
@@ -455,10 +485,12 @@ __device__ __forceinline__ int column_fill(const VolParams &V, const Column *__r
                 fov_planes(V, m, ic, c.Pa, c.Ga, 0, 0, lo, hi);   // z plays no part
                 ok = ok && i >= lo && i <= hi;
             }
-            ok = column_place<K2>(c, di, zc, nv, pad, ((sp.view - line_view0) * nu + u) * nvp, e) && ok;
+            const int line = (sp.view - line_view0) * nu + u;
+            const LineRange r = ranges[line];
+            ok = column_place<K2>(c, di, zc, nv, pad, line * nvp, nvp - pad - (int)r.from_end, (int)r.end - pad, e) && ok;
             e.w1 = upper_weight<SPL>(frac_of(pa));
             e.code |= row + 1;
-            e.line = GJP_CHECK_TAPS ? ((sp.view - line_view0) * nu + u) * nvp : 0;
+            e.line = GJP_CHECK_TAPS ? line * nvp : 0;
             e.length = GJP_CHECK_TAPS ? nvp : 0;
         }
     }
@@ -471,8 +503,9 @@ template <int K2, bool SPL, bool CAREFUL>
 __device__ __forceinline__ void column_gather(const float *__restrict__ lines, const VolParams &V,
                                               const ColumnView *__restrict__ cviews, const Column *__restrict__ cols,
                                               int nu, int nv, int nvp, int pad, int line_view0, int view_lo, int view_hi,
-                                              int m, int i, int a0, int zc, ColumnEntry *__restrict__ tab,
-                                              ColumnSpan *__restrict__ spans, float2 (&acc)[kStrip][K2])
+                                              int m, int i, int a0, int zc, const LineRange *__restrict__ ranges,
+                                              ColumnEntry *__restrict__ tab, ColumnSpan *__restrict__ spans,
+                                              float2 (&acc)[kStrip][K2])
 {
     const int lane16 = (int)(threadIdx.x & 31) - 16;
     for (int vb = view_lo; vb < view_hi; vb += 32) {
@@ -482,7 +515,7 @@ __device__ __forceinline__ void column_gather(const float *__restrict__ lines, c
         const int total = column_spans(cviews, nu, vb, view_hi, i, a0, spans, start, any);
         for (int q0 = 0; q0 < total; q0 += 32) {
             __syncwarp();                                // records written; every lane has read the last table
-            const int cnt = column_fill<K2, SPL>(V, cols, nu, nv, nvp, pad, line_view0, m, i, a0, zc, spans, start, any,
+            const int cnt = column_fill<K2, SPL>(V, cols, nu, nv, nvp, pad, line_view0, m, i, a0, zc, ranges, spans, start, any,
                                                     q0, total, tab);
             __syncwarp();
 #pragma unroll 1
@@ -523,7 +556,7 @@ constexpr int column_blocks(int K2) { return K2 == 1 ? 8 : K2 == 2 ? 6 : 4; }
 
 template <int K2, bool SPL>
 __global__ void __launch_bounds__(32 * kColWarps, column_blocks(K2)) gjp_adjoint_columns_kernel(
-    const float *__restrict__ lines, const unsigned *__restrict__ flag, VolParams V,
+    const float *__restrict__ lines, const unsigned *__restrict__ head, VolParams V,
     const ColumnView *__restrict__ cviews, const Column *__restrict__ cols, int nu, int nv, int nvp, int pad,
     int line_view0, int per_group, ColumnTiles T, float *__restrict__ vol)
 {
@@ -548,12 +581,13 @@ __global__ void __launch_bounds__(32 * kColWarps, column_blocks(K2)) gjp_adjoint
 #pragma unroll
         for (int p = 0; p < K2; ++p) acc[r][p] = make_float2(0.0f, 0.0f);
     ColumnEntry *tab = s_tab + 32 * warp;
-    if (__ldg(flag) == 0u)
+    const LineRange *ranges = line_ranges(head);
+    if (__ldg(head) == 0u)
         column_gather<K2, SPL, false>(lines, V, cviews, cols, nu, nv, nvp, pad, line_view0, view_lo, view_hi, m, i, a0,
-                                         zc, tab, s_spans + 32 * warp, acc);
+                                         zc, ranges, tab, s_spans + 32 * warp, acc);
     else
         column_gather<K2, SPL, true>(lines, V, cviews, cols, nu, nv, nvp, pad, line_view0, view_lo, view_hi, m, i, a0,
-                                        zc, tab, s_spans + 32 * warp, acc);
+                                        zc, ranges, tab, s_spans + 32 * warp, acc);
     const long long sm = m == 0 ? V.s[0] : V.s[1], sa = m == 0 ? V.s[1] : V.s[0];
     const int z0 = zc + lane;
     float *out = vol + (long long)i * sm + (long long)a0 * sa + z0;
@@ -571,7 +605,7 @@ __global__ void __launch_bounds__(32 * kColWarps, column_blocks(K2)) gjp_adjoint
 
 struct ColumnJob {
     const float *lines;
-    const unsigned *flag;
+    const unsigned *head;
     VolParams V;
     const ColumnForm *form;
     const gjp_geometry *g;
@@ -603,7 +637,7 @@ template <int K2> cudaError_t launch_tiles(const ColumnJob &j)
     const int per = (longest + groups - 1) / groups;
     const dim3 grid((unsigned)tiles, (unsigned)((longest + per - 1) / per));
     auto kern = j.g->weight == GJP_WEIGHT_SPL ? gjp_adjoint_columns_kernel<K2, true> : gjp_adjoint_columns_kernel<K2, false>;
-    kern<<<grid, 32 * kColWarps, 0, j.s>>>(j.lines, j.flag, V, j.form->d_views, j.form->d_cols, j.g->nu, j.g->nv, j.nvp,
+    kern<<<grid, 32 * kColWarps, 0, j.s>>>(j.lines, j.head, V, j.form->d_views, j.form->d_cols, j.g->nu, j.g->nv, j.nvp,
                                            j.pad, j.view0, per, T, j.vol);
     return cudaGetLastError();
 }
@@ -648,12 +682,13 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
     const int pad = line_pad(K2, form.pitch), nvp = line_length(g.nv, pad);
     const size_t line_bytes = (size_t)g.nu * nvp * sizeof(float);
     const int most = (int)std::max<size_t>(1, std::min<size_t>((size_t)g.n_views, (512ull << 20) / line_bytes));
+    const size_t head_bytes = (kHeadBytes + sizeof(LineRange) * (size_t)most * g.nu + 255) / 256 * 256;
     void *ws = nullptr;
-    const gjp_status got = workspace_alloc((size_t)most * line_bytes + 256, s, &ws);
+    const gjp_status got = workspace_alloc(head_bytes + (size_t)most * line_bytes, s, &ws);
     if (got != GJP_OK) return got;
     ColumnJob j;
-    j.flag = static_cast<unsigned *>(ws);
-    float *lines = reinterpret_cast<float *>(static_cast<char *>(ws) + 256);
+    j.head = static_cast<unsigned *>(ws);
+    float *lines = reinterpret_cast<float *>(static_cast<char *>(ws) + head_bytes);
     j.lines = lines;
     j.V = V;
     j.form = &form;
@@ -663,10 +698,10 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
     j.vol = vol;
     j.s = s;
     cudaError_t e = cudaStreamWaitEvent(s, form.ready, 0);       // the records, written on another stream perhaps
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, sizeof(unsigned), s);
     for (int v0 = 0; v0 < g.n_views && e == cudaSuccess; v0 += most) {
         j.view0 = v0;
         j.n_views = std::min(most, g.n_views - v0);
+        if ((e = cudaMemsetAsync(ws, 0, head_bytes, s)) != cudaSuccess) break;
         const dim3 tg((unsigned)((g.nu + 31) / 32), (unsigned)((nvp + 31) / 32), (unsigned)j.n_views);
         gjp_lines_kernel<<<tg, dim3(32, kTrRows), 0, s>>>(proj, V, form.d_cols, g.nu, g.nv, nvp, pad, v0, lines,
                                                           static_cast<unsigned *>(ws));

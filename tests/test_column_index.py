@@ -37,7 +37,7 @@ static void sweep(const long long *r, int n_cols, int nx, int ny, int nz, int nv
         for (int i = 0; i < nm; ++i)
             for (int zc = 0; zc < nz; zc += chunk_of(K2)) {
                 ColumnEntry e;
-                if (!column_place<K2>(c, i - ((nm - 1) >> 1), zc, nv, pad, line, e)) continue;
+                if (!column_place<K2>(c, i - ((nm - 1) >> 1), zc, nv, pad, line, 0, nv, e)) continue;
                 ++out[2];
                 for (int lane = 0; lane < 32; lane += 31) {
                     unsigned pos = column_position(e, lane - 16);
