@@ -331,7 +331,8 @@ gjp_status gjp_adjoint(const float *d_proj, const gjp_geometry *g, int64_t nx, i
  * to z in every view, rays driven by x or y, the grid in front of the
  * source, neighbouring rows 0.26 to 3 voxels apart inside the grid) on grids
  * with z lines of about 100 voxels or more, from 2^24 view-voxels (views x
- * voxels) on, and COMBINE otherwise.  The
+ * voxels) on, whose rows cover the z lines or a large part of them, and
+ * COMBINE otherwise.  The
  * column form gathers: each voxel sums the rays of the detector columns that
  * pass it, and is added to memory once per driving axis and group of views.
  * It reads a transposed copy of the projections, allocated on `stream` from

@@ -262,7 +262,7 @@ const ColumnForm *get_columns(const gjp_geometry *gc, gjp_cache_entry &e, const 
     char *d = nullptr;
     try {
         ColumnPlan plan;
-        if (!column_plan(*g, n, h, o, plan)) {
+        if (!column_plan(*g, n, h, o, plan) || !columns_pay(plan.extent, n, g->n_views)) {
             f.state = ColumnForm::kNone;
             return nullptr;
         }
@@ -291,8 +291,7 @@ const ColumnForm *get_columns(const gjp_geometry *gc, gjp_cache_entry &e, const 
         f.d_views = reinterpret_cast<ColumnView *>(d);
         f.d_cols = cols;
         f.ready = ready;
-        f.pitch = plan.pitch;
-        f.pitch_max = plan.pitch_max;
+        f.extent = plan.extent;
         f.state = ColumnForm::kReady;
         return &f;
     } catch (const std::bad_alloc &) {
@@ -2344,7 +2343,7 @@ gjp_status gjp_adjoint_ex(const float *d_proj, const gjp_geometry *g, int64_t nx
     if (path == GJP_PATH_AUTO && columns_pay(n, g->n_views)) {
         const RelaxedCapture relaxed;
         const ColumnForm *form = get_columns(g, *entry, n, h, o, s);
-        if (form && columns_pay(*form, n, g->n_views)) {
+        if (form) {
             st = adjoint_columns(d_proj, make_vol(n, h, g->fov), *form, *g, d_volume, s);
             if (st == GJP_OK || st == GJP_ERR_CUDA) return st;
         }

@@ -104,10 +104,17 @@ struct ColumnView {
 };
 constexpr int kMaxColumns = 1 << 22;
 // Host: the views that each driving axis has columns of, and the least and
-// the largest row pitch (voxels).
+// the largest row pitch (voxels).  The middle column of each view on the
+// grid's centre plane gives the sums over the views of the z voxels that the
+// detector's rows cover and of the z chunks that these meet, the mean pitch,
+// and whether every view covers the whole z range.
+struct ColumnExtent {
+    double pitch = 0.0, pitch_max = 0.0, pitch_mean = 0.0, covered = 0.0, chunks = 0.0;
+    bool whole = true;
+};
 struct ColumnPlan {
     std::vector<ColumnView> views[2];
-    double pitch = 0.0, pitch_max = 0.0;
+    ColumnExtent extent;
 };
 // The column form on a device (one allocation, at d_views).
 struct ColumnForm {
@@ -117,7 +124,7 @@ struct ColumnForm {
     Column *d_cols = nullptr;                 // [view][iu]
     cudaEvent_t ready = nullptr;              // both are written
     std::vector<int> view_ids[2];
-    double pitch = 0.0, pitch_max = 0.0;
+    ColumnExtent extent;
 };
 
 struct gjp_cache_entry {
@@ -241,7 +248,7 @@ bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], c
 cudaError_t write_columns(const ViewParams *views, const VolParams &V, const gjp_geometry &g, Column *cols,
                           cudaStream_t s);
 bool columns_pay(const int64_t n[3], int n_views, double pitch = 1.0);
-bool columns_pay(const ColumnForm &form, const int64_t n[3], int n_views);
+bool columns_pay(const ColumnExtent &extent, const int64_t n[3], int n_views);
 gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnForm &form, const gjp_geometry &g,
                            float *vol, cudaStream_t s);
 // The forward's column form: whether it covers a scan, whether it is the

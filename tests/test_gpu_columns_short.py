@@ -60,3 +60,28 @@ def test_rows_of_half_the_height(gjp, shift, sign):
     vg, cg = _scan((108, 100, 512), 4, 60, 130, 4.0, 2.0, shift, sign)
     d, g = _check(gjp, vg, cg)
     assert takes_columns(gjp, d, g, vg)
+
+
+def _ms(f):
+    best = 1e9
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        a.record()
+        for _ in range(3):
+            f()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) / 3)
+    return best
+
+
+@pytest.mark.parametrize("nv,pitch", [(16, 1.0), (64, 1.0), (61, 0.5), (24, 2.0)])
+def test_few_rows_cost_no_more_than_the_scatter(gjp, nv, pitch):
+    vg, cg = _scan((256, 256, 256), 4, 256, nv, 8.0, pitch, 0.0, 1)
+    cg = synth.ConeGeometry(*(np.tile(x, (23, 1)) for x in (cg.src, cg.det_origin, cg.det_u, cg.det_v)), cg.nu, cg.nv)
+    g = gjp.Geometry.from_cone(cg)
+    y = torch.randn(g.proj_shape, device="cuda")
+    out = torch.empty(vg.n, device="cuda")
+    t = [_ms(lambda: gjp.adjoint(y, g, vg.n, vg.h, out=out, path=p)) for p in ("auto", "combine")]
+    assert t[0] <= 1.3 * t[1], t
