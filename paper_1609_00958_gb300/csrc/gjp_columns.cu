@@ -334,17 +334,16 @@ template <bool SPL> __device__ __forceinline__ float2 shape(float2 e)
 }
 
 // Debug build (GJP_CHECK_TAPS): where a lane loads `n` elements of entry e's
-// line from; loads that would leave the line are recorded and read its first
-// elements instead (a line is longer than any n).  The element itself, and
-// free, in the production build.
-__device__ __forceinline__ int checked_element(const ColumnEntry &e, unsigned position, int n)
+// line of nvp elements from; loads that would leave the line are recorded and
+// read its first elements instead (a line is longer than any n).  The element
+// itself, and free, in the production build.
+__device__ __forceinline__ int checked_element(const ColumnEntry &e, long long position, int n, int nvp)
 {
     const int k = column_element(position);
     if (!GJP_CHECK_TAPS) return k;
-    const int in_line = e.base + k - e.line;
-    const bool ok = in_line >= 0 && in_line + n <= e.length;
+    const bool ok = k >= e.line && k + n <= e.line + nvp;
     if (!ok) atomicOr(&g_gjp_tap_fault, 1u);
-    return ok ? k : e.line - e.base;
+    return ok ? k : e.line;
 }
 
 // The same for the taps z0 and z0 + 1 of a forward line of nz voxels with its
@@ -362,36 +361,33 @@ __device__ __forceinline__ int checked_line_tap(int z0, int nz, int edge)
 // above z - 1; N = 0: the first n above z - 1.  CAREFUL keeps a ray out of
 // reach from contributing 0 x inf.
 template <int K2, int N, bool SPL, bool CAREFUL>
-__device__ __forceinline__ void column_sums(const float *__restrict__ lines, const ColumnEntry &e, int lane16, int n,
+__device__ __forceinline__ void column_sums(const float *__restrict__ lines, const ColumnEntry &e, int lane, int n, int nvp,
                                             float2 (&q)[K2])
 {
-    const float *line = lines + e.base;
-    unsigned pos = column_position(e, lane16);
-    const unsigned half = column_half(e);
-    const float B = e.pitch;
+    long long pos = column_position(e, lane);
+    const long long half = column_half(e);
+    const float B = e.pitch, b = B * 2.3283064365386963e-10f;            // per 2^-32 of a ray
 #pragma unroll
     for (int p = 0; p < K2; ++p) {
         float2 w[3], y[3];
-        float f[2];
+        float f[2];                                                      // past the ray, in 2^-32 rays
         const float *at[2];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-            const unsigned x = s ? pos + half : pos;
-            at[s] = line + checked_element(e, x, N > 0 ? N : n);
-            f[s] = __uint_as_float((x & 0x7FFFFFu) | 0x3F800000u);          // 1 + fraction
+            at[s] = lines + checked_element(e, pos, N > 0 ? N : n, nvp);
+            f[s] = __uint2float_rn((unsigned)pos);
+            pos += half;
         }
-        pos += (unsigned)e.inv;
-        // what is left of the ray's step to the next ray (exact), in rays
-        const float2 F = make_float2(f[0], f[1]), m1 = make_float2(-1.0f, -1.0f);
-        const float2 left = __ffma2_rn(F, m1, make_float2(2.0f, 2.0f));
         if (N == 2) {
-            const float2 past = __fadd2_rn(F, m1);
-            w[0] = make_float2(fma_sat(-past.x, B, 1.0f), fma_sat(-past.y, B, 1.0f));
-            w[1] = make_float2(fma_sat(-left.x, B, 1.0f), fma_sat(-left.y, B, 1.0f));
+            w[0] = make_float2(fma_sat(-f[0], b, 1.0f), fma_sat(-f[1], b, 1.0f));
+            w[1] = make_float2(fma_sat(f[0], b, 1.0f - B), fma_sat(f[1], b, 1.0f - B));
         } else if (N == 3) {
-            w[0] = __fmul2_rn(left, make_float2(B, B));
-            w[1] = make_float2(1.0f - fabsf(__fmaf_rn(left.x, B, B - 1.0f)), 1.0f - fabsf(__fmaf_rn(left.y, B, B - 1.0f)));
-            w[2] = make_float2(fma_sat(-left.x, B, 2.0f - 2.0f * B), fma_sat(-left.y, B, 2.0f - 2.0f * B));
+            const float2 F = make_float2(f[0], f[1]), mb = make_float2(-b, -b);
+            const float c = B - 1.0f;
+            w[0] = __ffma2_rn(F, mb, make_float2(B, B));
+            const float2 t = __fadd2_rn(w[0], make_float2(c, c));
+            w[1] = make_float2(1.0f - fabsf(t.x), 1.0f - fabsf(t.y));
+            w[2] = make_float2(fma_sat(c, -2.0f, -w[0].x), fma_sat(c, -2.0f, -w[0].y));
         }
         if (N > 0) {
 #pragma unroll
@@ -407,7 +403,7 @@ __device__ __forceinline__ void column_sums(const float *__restrict__ lines, con
 #pragma unroll
             for (int j = 1; j < N; ++j) q[p] = __ffma2_rn(w[j], y[j], q[p]);
         } else {
-            float2 d = make_float2(__fmaf_rn(left.x, B, -1.0f), __fmaf_rn(left.y, B, -1.0f));
+            float2 d = __ffma2_rn(make_float2(f[0], f[1]), make_float2(-b, -b), make_float2(B - 1.0f, B - 1.0f));
             float2 sum = make_float2(0.0f, 0.0f);
             for (int j = 0; j < n; ++j) {
                 const float2 v = shape<SPL>(make_float2(__saturatef(1.0f - fabsf(d.x)), __saturatef(1.0f - fabsf(d.y))));
@@ -506,7 +502,6 @@ __device__ __forceinline__ int column_fill(const VolParams &V, const Column *__r
             e.w1 = upper_weight<SPL>(frac_of(pa));
             e.code |= row + 1;
             e.line = GJP_CHECK_TAPS ? line * nvp : 0;
-            e.length = GJP_CHECK_TAPS ? nvp : 0;
         }
     }
     const unsigned mask = __ballot_sync(0xffffffffu, ok);
@@ -522,7 +517,7 @@ __device__ __forceinline__ void column_gather(const float *__restrict__ lines, c
                                               ColumnEntry *__restrict__ tab, ColumnSpan *__restrict__ spans,
                                               float2 (&acc)[kStrip][K2])
 {
-    const int lane16 = (int)(threadIdx.x & 31) - 16;
+    const int lane = (int)(threadIdx.x & 31);
     for (int vb = view_lo; vb < view_hi; vb += 32) {
         int start;
         bool any;
@@ -538,9 +533,9 @@ __device__ __forceinline__ void column_gather(const float *__restrict__ lines, c
                 const ColumnEntry e = tab[k];
                 const int n = e.code >> 4;
                 float2 q[K2];
-                if (n == 2) column_sums<K2, 2, SPL, CAREFUL>(lines, e, lane16, n, q);
-                else if (n == 3) column_sums<K2, 3, SPL, CAREFUL>(lines, e, lane16, n, q);
-                else column_sums<K2, 0, SPL, CAREFUL>(lines, e, lane16, n, q);
+                if (n == 2) column_sums<K2, 2, SPL, CAREFUL>(lines, e, lane, n, nvp, q);
+                else if (n == 3) column_sums<K2, 3, SPL, CAREFUL>(lines, e, lane, n, nvp, q);
+                else column_sums<K2, 0, SPL, CAREFUL>(lines, e, lane, n, nvp, q);
                 const float2 w1 = make_float2(e.w1, e.w1), w0 = make_float2(1.0f - e.w1, 1.0f - e.w1);
                 const auto rows = [&](auto r) {           // rows r - 1 and r of the tile
                     constexpr int R = decltype(r)::value;

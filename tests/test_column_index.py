@@ -40,10 +40,10 @@ static void sweep(const long long *r, int n_cols, int nx, int ny, int nz, int nv
                 if (!column_place<K2>(c, i - ((nm - 1) >> 1), zc, nv, pad, line, 0, nv, e)) continue;
                 ++out[2];
                 for (int lane = 0; lane < 32; lane += 31) {
-                    unsigned pos = column_position(e, lane - 16);
-                    for (int p = 0; p < K2; ++p, pos += (unsigned)e.inv)
-                        for (int s = 0; s < 2; ++s) {
-                            const long long first = (long long)e.base + column_element(s ? pos + column_half(e) : pos);
+                    long long pos = column_position(e, lane);
+                    for (int p = 0; p < K2; ++p)
+                        for (int s = 0; s < 2; ++s, pos += column_half(e)) {
+                            const long long first = column_element(pos);
                             if (first - line < out[0]) out[0] = first - line;
                             if (first + (e.code >> 4) - 1 - line > out[1]) out[1] = first + (e.code >> 4) - 1 - line;
                         }
