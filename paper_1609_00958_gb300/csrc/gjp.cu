@@ -322,14 +322,14 @@ __global__ void __launch_bounds__(kTileV * kTileU, PAIRS ? 4 : 5) gjp_forward_de
         forward_ray<T, int, SPL, PAIRS, kDeepPlanes<PAIRS>>(vol, V, views + view, nu, nv, iu, iv, act, (int)threadIdx.y, pairs);
 }
 
-bool takes_columns(const gjp_geometry *gc, gjp_cache_entry *e, const int64_t n[3], const double h[3], gjp_dtype dt,
-                   const void *vol)
+bool takes_columns(const gjp_geometry *gc, gjp_cache_entry *e, const int64_t n[3], const double h[3], const double o[3],
+                   gjp_dtype dt, const void *vol)
 {
     if (!forward_columns_pay(n, gc->nu, gc->nv, gc->n_views, dt, vol)) return false;
-    if (!e) return column_rays(*gc, h);
+    if (!e) return column_rays(*gc, n, h, o);
     gjp_geometry *g = const_cast<gjp_geometry *>(gc);
     std::lock_guard<std::mutex> lock(g->mu);
-    if (e->column_rays < 0) e->column_rays = column_rays(*g, h) ? 1 : 0;
+    if (e->column_rays < 0) e->column_rays = column_rays(*g, n, h, o) ? 1 : 0;
     return e->column_rays == 1;
 }
 
@@ -1935,7 +1935,7 @@ gjp_status forward_typed(const void *d_volume, gjp_dtype dt, const int64_t n[3],
         }
         if (path == GJP_PATH_SLAB) return GJP_ERR_UNSUPPORTED;
     }
-    if (path == GJP_PATH_AUTO && takes_columns(&g, &entry, n, h, dt, d_volume)) {
+    if (path == GJP_PATH_AUTO && takes_columns(&g, &entry, n, h, o, dt, d_volume)) {
         const GatherShape sh{g.nu, g.nv, g.n_views, g.tile_u, launch_view_group(g, V.n), g.weight == GJP_WEIGHT_SPL};
         return forward_columns(d_volume, dt, V, table, sh, proj, s) == cudaSuccess ? GJP_OK : GJP_ERR_CUDA;
     }
@@ -2257,7 +2257,7 @@ gjp_status gjp_forward_noalloc(const void *d_volume, gjp_dtype dtype, int64_t nx
     const VolParams V = make_vol(n, h, g->fov);
     const bool i32 = fits_int32(n);
     cudaError_t e = cudaSuccess;
-    if (takes_columns(g, nullptr, n, h, dtype, d_volume)) {
+    if (takes_columns(g, nullptr, n, h, o, dtype, d_volume)) {
         const GatherShape sh{g->nu, g->nv, g->n_views, g->tile_u, launch_view_group(*g, V.n), g->weight == GJP_WEIGHT_SPL};
         return forward_columns(d_volume, dtype, V, d_table, sh, d_proj, s) == cudaSuccess ? GJP_OK : GJP_ERR_CUDA;
     }

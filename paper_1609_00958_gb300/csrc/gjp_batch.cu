@@ -332,7 +332,7 @@ gjp_status gjp_batch_create(const gjp_problem *problems, int count, gjp_batch **
         const int tu = valid_tile(q.geometry->tile_u) ? q.geometry->tile_u : 4;
         shape_problem(P, tu, launch_view_group(*q.geometry, n), q.geometry->n_views);
         planes[p] = (int)std::max(n[0], std::max(n[1], n[2]));
-        columns[p] = takes_columns(q.geometry, entry, n, h, q.dtype, q.d_volume) ? 1 : 0;
+        columns[p] = takes_columns(q.geometry, entry, n, h, o, q.dtype, q.d_volume) ? 1 : 0;
     }
     // queue order: problems with the longest rays (most planes per item) first
     std::vector<int> order(count);

@@ -13,8 +13,15 @@
 
 namespace gjp_detail {
 
-// Fraction bits of the row pitch B in Column (z positions have 32).
-constexpr int kPitchBits = 40;
+// Fraction bits of the row pitch B in Column (z positions have 32).  The
+// pitch is multiplied by up to kMostRows / 2 rows and as many planes: 46 bits
+// keep 1024 planes of 32768 rows to 2^-24 voxel, what a ray's own increment
+// per plane has.  Rows spread over kMostSpread voxels at most, so that their
+// product fits 64 bits.
+constexpr int kPitchBits = 46;
+constexpr float kPitchScale = (float)(1LL << kPitchBits), kPitchUnit = 1.0f / kPitchScale;
+constexpr int kMostRows = 1 << 15;
+constexpr double kMostSpread = 32768.0;
 
 // One detector column of one view: the (x, y) path its rays share and their
 // z positions, in fixed point (32 fraction bits; the pitch kPitchBits).
@@ -61,11 +68,11 @@ GJP_HD long long column_fixed(float x)             // round(x 2^32)
 template <int K2>
 GJP_HD bool column_place(const Column &c, int di, int zc, int nv, int pad, int line, int first, int end, ColumnEntry &e)
 {
-    const float inv32 = 2.3283064365386963e-10f, invp = 9.094947017729282e-13f;   // 2^-32, 2^-kPitchBits
+    const float inv32 = 2.3283064365386963e-10f, invp = kPitchUnit;                // 2^-32, 2^-kPitchBits
     const long long bs = c.Y0 + (long long)di * c.Y1;
     const long long bq = bs < 0 ? -bs : bs;
     const float b = (float)bq * invp;
-    const float b_lo = (float)(bq - (long long)(b * 1099511627776.0f)) * invp;     // exact: b has 24 bits
+    const float b_lo = (float)(bq - (long long)(b * kPitchScale)) * invp;     // exact: b has 24 bits
     const float x = 1.0f / b;
     const float x_lo = fmaf(-b, x, 1.0f) * x - b_lo * x * x;           // 1 / B = x + x_lo
     const int n = b >= 1.0f ? 2 : (int)ceilf(2.0001f * x);

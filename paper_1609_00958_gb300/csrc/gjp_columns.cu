@@ -72,11 +72,12 @@ static void view_direction(const gjp_geometry &g, int k, const double h[3], doub
     }
 }
 
-// Whether the forward's column form covers a scan: detector rows along z in
-// every view and slopes along z below 1/2.
-bool column_rays(const gjp_geometry &g, const double h[3])
+// Whether the forward's column form covers a scan on a grid: detector rows
+// along z in every view, slopes along z below 1/2, and rows that spread over
+// kMostSpread voxels at most on the centre plane.
+bool column_rays(const gjp_geometry &g, const int64_t n[3], const double h[3], const double o[3])
 {
-    if (g.nv > (1 << 15)) return false;
+    if (g.nv > kMostRows) return false;
     for (int k = 0; k < g.n_views; ++k)
         if (g.dv[3 * k] != 0.0 || g.dv[3 * k + 1] != 0.0) return false;
     const double cu = 0.5 * (g.nu - 1), cv = 0.5 * (g.nv - 1);
@@ -84,8 +85,12 @@ bool column_rays(const gjp_geometry &g, const double h[3])
         double r0[3], ru[3], change;
         int changes;
         view_direction(g, k, h, r0, ru);
-        const double rise = std::fabs(r0[2]) + cu * std::fabs(ru[2]) + cv * std::fabs(g.dv[3 * k + 2] / h[2]);
-        if (!(rise < 0.49 * least_lateral(r0, ru, cu, changes, change))) return false;
+        const double pv = std::fabs(g.dv[3 * k + 2] / h[2]), least = least_lateral(r0, ru, cu, changes, change);
+        if (!(std::fabs(r0[2]) + cu * std::fabs(ru[2]) + cv * pv < 0.49 * least)) return false;
+        for (int m = 0; m < 2; ++m) {
+            const double away = std::fabs((g.src[3 * k + m] - o[m]) / h[m] - 0.5 * (double)(n[m] - 1));
+            if (!(g.nv * pv * away < kMostSpread * least)) return false;
+        }
     }
     return true;
 }
@@ -97,7 +102,7 @@ bool column_rays(const gjp_geometry &g, const double h[3])
 // and a grid on which the float32 column search is good to half its margin.
 bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], const double o[3], ColumnPlan &plan)
 {
-    if (g.n_views > 65535 || (int64_t)g.n_views * g.nu > kMaxColumns || g.nv > (1 << 15) ||
+    if (g.n_views > 65535 || (int64_t)g.n_views * g.nu > kMaxColumns || g.nv > kMostRows ||
         (int64_t)g.nu * (g.nv + 4096) > (1 << 27))
         return false;
     for (int a = 0; a < 3; ++a)
@@ -170,6 +175,7 @@ bool column_plan(const gjp_geometry &g, const int64_t n[3], const double h[3], c
         x.pitch_mean += std::fabs(t * pv) / g.n_views;
         rows[k] = {s[2] + t * r0[2] - half, s[2] + t * r0[2] + half};
     }
+    if (!(g.nv * x.pitch_max < kMostSpread)) return false;
     const double top = (double)(n[2] - 1), chunk = chunk_of(column_pairs((int)n[2], x.pitch));
     for (const auto &r : rows) {
         const double lo = std::max(0.0, r.first), hi = std::min(top, r.second);
@@ -204,14 +210,13 @@ __device__ __forceinline__ Column make_column(const ViewParams &vp, const VolPar
     const f2 dg = f2_div({vp.rh[8], vp.rl[8]}, rm, inv);                            // d(rt_z) / dv
     const int nm = m == 0 ? V.n[0] : V.n[1];
     const f2 y0 = f2_shift(dq, 0.0f, dg, (float)R.ic - 0.5f * (float)(nm - 1));
-    const float scale = 1099511627776.0f;   // 2^kPitchBits
     Column c;
     c.Pa = R.Pa;
     c.Ga = R.Ga;
     c.Z0 = R.Pb;
     c.Z1 = R.Gb;
-    c.Y0 = __float2ll_rn(y0.hi * scale) + __float2ll_rn(y0.lo * scale);
-    c.Y1 = __float2ll_rn(dg.hi * scale) + __float2ll_rn(dg.lo * scale);
+    c.Y0 = __float2ll_rn(y0.hi * kPitchScale) + __float2ll_rn(y0.lo * kPitchScale);
+    c.Y1 = __float2ll_rn(dg.hi * kPitchScale) + __float2ll_rn(dg.lo * kPitchScale);
     c.m = m;
     c.pad = 0;
     return c;
@@ -282,7 +287,6 @@ __global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__
     }
     __syncthreads();
     const float inv = 2.3283064365386963e-10f;                       // 2^-32
-    const float vs = 9.094947017729282e-13f;                         // 2^-kPitchBits
     bool bad = false;
 #pragma unroll
     for (int k = threadIdx.y; k < 32; k += kTrRows) {
@@ -294,7 +298,7 @@ __global__ void __launch_bounds__(32 * kTrRows) gjp_lines_kernel(const float *__
         const int r = p - pad;
         const float v = (float)(down ? nv - 1 - r : r) - 0.5f * (float)(nv - 1);
         const float ga = ha * (__ll2float_rn(c->Ga) * inv);
-        const float gb = V.h[2] * __fmaf_rn(v, __ll2float_rn(c->Y1) * vs, __ll2float_rn(c->Z1) * inv);
+        const float gb = V.h[2] * __fmaf_rn(v, __ll2float_rn(c->Y1) * kPitchUnit, __ll2float_rn(c->Z1) * inv);
         const float y = tile[threadIdx.x][k] * sqrtf(hm * hm + ga * ga + gb * gb);
         bad = bad || !(fabsf(y) <= 3.402823466e38f);
         const size_t line = (size_t)blockIdx.z * nu + u;

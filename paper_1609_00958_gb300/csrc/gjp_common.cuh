@@ -197,8 +197,8 @@ bool pairs_pay(int n_views, const int64_t n[3]);
 // Whether gjp_forward (AUTO), gjp_forward_noalloc and batches project a problem
 // with the column form of the forward (gjp.cu; e: the geometry's entry for
 // the grid, or null).  All three ask here, so that their results are the same.
-bool takes_columns(const gjp_geometry *g, gjp_cache_entry *e, const int64_t n[3], const double h[3], gjp_dtype dt,
-                   const void *vol);
+bool takes_columns(const gjp_geometry *g, gjp_cache_entry *e, const int64_t n[3], const double h[3], const double o[3],
+                   gjp_dtype dt, const void *vol);
 // Writes the z-paired copy (4 bytes per voxel) of a bfloat16 or float16 volume.
 cudaError_t write_zpairs16(const void *vol, gjp_dtype dt, const int64_t n[3], void *out, cudaStream_t s);
 // Texture families (gjp_texture.cu): forward through the texture unit, and
@@ -253,7 +253,7 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
                            float *vol, cudaStream_t s);
 // The forward's column form: whether it covers a scan, whether it is the
 // faster one for a problem that it covers, and its launch.
-bool column_rays(const gjp_geometry &g, const double h[3]);
+bool column_rays(const gjp_geometry &g, const int64_t n[3], const double h[3], const double o[3]);
 bool forward_columns_pay(const int64_t n[3], int nu, int nv, int n_views, gjp_dtype dt, const void *vol);
 cudaError_t forward_columns(const void *vol, gjp_dtype dt, const VolParams &V, const ViewParams *table,
                             const GatherShape &sh, float *proj, cudaStream_t s);

@@ -52,6 +52,17 @@ static void sweep(const long long *r, int n_cols, int nx, int ny, int nz, int nv
     }
 }
 
+extern "C" int pitch_bits() { return kPitchBits; }
+
+// position of the chunk's first voxel above the line's first ray, in rays (N > 2: of the voxel below it)
+extern "C" double first_position(const long long *r, int nm, int i, int zc, int nv, int *rays)
+{
+    ColumnEntry e;
+    column_place<4>(Column{0, 0, r[0], r[1], r[2], r[3], (int)r[4], 0}, i - ((nm - 1) >> 1), zc, nv, 0, 0, 0, nv, e);
+    *rays = e.code >> 4;
+    return (double)(e.pos >> 32) + (double)(e.pos & 0xffffffffLL) / 4294967296.0;
+}
+
 extern "C" void sweep_scan(const long long *r, int n_cols, int nx, int ny, int nz, int nv, int k2, double pitch, long long *out)
 {
     switch (k2) {
@@ -76,7 +87,7 @@ def lib(tmp_path_factory):
     return ctypes.CDLL(str(so))
 
 
-def _columns(vg, cg):
+def _columns(vg, cg, bits):
     """Records Z0, Z1, Y0, Y1, m of every (view, column), and the least pitch on the grid's end planes."""
     n, h, o = (np.array(v, float) for v in (vg.n, vg.h, vg.origin))
     src = (cg.src - o) / h
@@ -89,14 +100,14 @@ def _columns(vg, cg):
     nm = n[m]
     t = (np.floor((nm - 1) / 2) - sm) / rm
     ends = np.abs(np.stack([(0 - sm) / rm, (nm - 1 - sm) / rm]) * dv[:, 2][:, None])
-    z, y = float(1 << 32), float(1 << 40)
+    z, y = float(1 << 32), float(1 << bits)
     rec = [(src[:, 2][:, None] + t * r[..., 2]) * z, r[..., 2] / rm * z, t * dv[:, 2][:, None] * y, dv[:, 2][:, None] / rm * y]
     rec = np.stack([np.rint(a).astype(np.int64) for a in rec] + [m.astype(np.int64)], -1)
     return np.ascontiguousarray(rec.reshape(-1, 5)), float(ends.min())
 
 
 def _sweep(lib, vg, cg, k2):
-    rec, pitch = _columns(vg, cg)
+    rec, pitch = _columns(vg, cg, lib.pitch_bits())
     out = (ctypes.c_longlong * 4)()
     lib.sweep_scan(rec.ctypes.data_as(ctypes.c_void_p), len(rec), *[int(v) for v in vg.n], cg.nv, k2, ctypes.c_double(pitch), out)
     return pitch, list(out)
@@ -162,3 +173,25 @@ def test_loads_stay_in_their_lines_over_the_range(lib):
             cg.det_origin, cg.det_v = cg.det_origin + (nv - 1) * cg.det_v, -cg.det_v
         entries += _check(lib, VolumeGeometry.centred(n, (1.0, 1.0, float(rng.uniform(0.6, 1.6)))), cg)
     assert entries > 100000
+
+
+def test_positions_on_a_tall_detector(lib):
+    """Many fine rows far from the centre plane: positions within 4e-7 voxel of float64's (increments per plane hold
+    2^-33 voxel, times 512 planes, and as much for the rows; with 40 fraction bits of the rows' distance 2e-6)."""
+    n, nv = (1024, 24, 4096), 12000
+    vg, cg = VolumeGeometry.centred(n), _cone(n, 2, 3, nv, 4.0, 0.33)
+    rec, _ = _columns(vg, cg, lib.pitch_bits())
+    lib.first_position.restype = ctypes.c_double
+    src = cg.src - np.array(vg.origin)
+    for col, row in enumerate(rec):
+        k, u = divmod(col, cg.nu)
+        r = cg.det_origin[k] + u * cg.det_u[k] - cg.src[k]                 # to row 0, the lowest one
+        m = int(row[4])
+        for i in (0, 100, n[m] // 2, n[m] - 1):
+            t = (i - src[k, m]) / r[m]
+            low, pitch = src[k, 2] + t * r[2], t * cg.det_v[k, 2]
+            for zc in (0, 256, 2048, 3840):
+                rays = ctypes.c_int()
+                got = lib.first_position(row.ctypes.data_as(ctypes.c_void_p), n[m], i, zc, nv, ctypes.byref(rays))
+                below = 1 if rays.value > 2 else 0                         # the element is counted one up there
+                assert abs((got - below) * pitch - (zc - below - low)) <= 4e-7, (col, i, zc)
