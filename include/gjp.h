@@ -209,8 +209,9 @@ typedef enum {
  * detector rows run along z (det_v parallel to z in every view, slopes
  * along z below 1/2) on grids of 112 to 1024 voxels along z, a multiple of
  * 4, with 32-bit offsets, a volume aligned to 4 voxels, more than 2^22 voxels
- * (16-bit storage: 2^25), enough columns and views to fill the GPU and line
- * and detector lengths that fill its warps: a block interpolates whole z
+ * (16-bit storage: 2^25), enough columns and views to fill the GPU, line
+ * and detector lengths that fill its warps, and enough of the detector's rows
+ * inside the grid: a block interpolates whole z
  * lines between the two rows of a plane once for all rays of a detector
  * column and samples them from shared memory.  It allocates nothing, and its
  * results agree with GATHER's to float32 rounding.
