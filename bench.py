@@ -291,8 +291,16 @@ _UNIT_SCALE = {"byte": 1.0, "kbyte": 1e3, "mbyte": 1e6, "gbyte": 1e9, "tbyte": 1
 # touches two transverse rows over the z-span of 32 neighbouring rays, 33 voxels
 # (132 bytes in float32: two 128-byte L1 lines and five 32-byte sectors; 66 bytes in
 # 16-bit storage: one or two lines, 1.5 on average).
+# The column forms: a warp-plane of the forward forms 32 voxels of a line from two rows (a
+# wavefront each, half of one in 16-bit storage), stores them (one) and reads two taps of 33
+# words (two); the adjoint's 32 voxels read two rays each.
 # A note names the binding resource where the unit's own fraction is not the largest.
 LIMIT_MODEL = {
+    "gjp_forward_columns_kernel<float": ("l1_wavefronts", "l1_wavefronts_pct", "L1 data-pipe wavefronts", 5.0, None),
+    "gjp_forward_columns_kernel<__nv_bfloat16": ("l1_wavefronts", "l1_wavefronts_pct", "L1 data-pipe wavefronts", 4.0,
+                                                 "issue slots bind first"),
+    "gjp_adjoint_columns_kernel<4": ("l1_wavefronts", "l1_wavefronts_pct", "L1 data-pipe wavefronts", 2.0,
+                                     "issue slots and dependent-instruction waits bind at 16 warps per SM"),
     "gjp_forward_kernel<float": ("l1_wavefronts", "l1_wavefronts_pct", "L1 data-pipe wavefronts", 2 * 2.0, None),
     "gjp_forward_kernel<__nv_bfloat16": ("l1_wavefronts", "l1_wavefronts_pct", "L1 data-pipe wavefronts",
                                          2 * 1.5, "z-paired taps: one 4-byte load per row; the L1 does not "
@@ -349,7 +357,9 @@ def ncu_summary(csv_path: str, views: int, command: str, n: int = 512, n_views: 
     return {"sources": _sources_hash(), "kernels": kernels,
             "capture": {"views": views, "of_views": n_views, "volume": n, "command": command,
                         "note": f"one ncu capture of the first {views} views (one view group) of the {n_views}-view "
-                                f"{n}^3 workload; DRAM bytes scaled x{n_views / views:g} to a full launch"}}
+                                f"{n}^3 workload; DRAM bytes scaled x{n_views / views:g} to a full launch (an upper "
+                                "bound for the column adjoint, which adds a voxel to memory once per group of up to "
+                                "64 MB of projections)"}}
 
 
 def ncu_record(kernel: str):
@@ -485,7 +495,7 @@ def run_gjp(args):
     alg_bytes = {
         "forward_f32": 4.0 * foot.sum() + proj_bytes,
         k16: 2.0 * foot.sum() + proj_bytes,
-        "adjoint_f32": 8.0 * foot.sum() + proj_bytes,    # read-modify-write of each touched voxel per view
+        "adjoint_f32": adjoint_bytes(vg, cg, foot, proj_bytes),
     }
 
     names = ["forward_f32", k16, "adjoint_f32"] + (["allreduce"] if world > 1 else [])
@@ -549,9 +559,11 @@ def run_gjp(args):
                 else "fallback", "unit": "GB/s",
                 "frac": round(kernels[dominant]["achieved_gbs"] / hbm, 4),
                 "frac_algorithmic": round(kernels[dominant]["achieved_gbs"] / hbm, 4),
-                "frac_note": "algorithmic bytes: per view, every voxel with a non-zero tap once (adjoint: read "
-                             "and written), summed over the views; views issued together share the L2, so the "
-                             "DRAM traffic is far lower (dram_frac)",
+                "frac_note": "algorithmic bytes of a forward: per view, every voxel with a non-zero tap once, summed "
+                             "over the views (views issued together share the L2, so the DRAM traffic is far lower, "
+                             "dram_frac); of a scatter adjoint: those read and written; of a column adjoint, which "
+                             "sums the views in registers: each voxel read and written once, the projections read, "
+                             "their transposed copy written and read",
                 "traffic": traffic,
                 "dram_frac": None if traffic is None else round(traffic / dmsec / 1e9 / hbm, 4),
                 "limiter": kernels[dominant].get("limiter")}
@@ -637,7 +649,8 @@ def c1_kernels(gjp, dev, reps: int = 200):
 
 def takes_columns(n, nu: int, nv: int, n_views: int, sixteen: bool) -> bool:
     """Whether AUTO projects with the forward's column form (the library's
-    forward_columns_pay rule; the benchmark's scans have their rows along z)."""
+    forward_columns_pay rule; the benchmark's scans have their rows along z
+    and inside the grid)."""
     nx, ny, nz = (int(v) for v in n)
     if nz % 4 or not 112 <= nz <= 1024 or nx * ny * nz + 2 * (ny * nz + nz + 1) >= 2147483647:
         return False
@@ -652,10 +665,20 @@ def takes_columns(n, nu: int, nv: int, n_views: int, sixteen: bool) -> bool:
     return voxels > 2 ** 22 and (cost <= 1.06 or (cost <= 1.16 and voxels >= 8.5e7))
 
 
+def adjoint_bytes(vg, cg, foot, proj_bytes: float) -> float:
+    """Bytes that one AUTO adjoint cannot do without: a scatter reads and
+    writes each touched voxel per view; the column form each voxel once, and
+    it reads the projections and writes and reads a transposed copy."""
+    if adjoint_launches(vg, cg) == 1:
+        return 8.0 * float(foot.sum()) + proj_bytes
+    return 8.0 * float(np.prod([int(v) for v in vg.n])) + 3.0 * proj_bytes
+
+
 def adjoint_launches(vg, cg) -> int:
-    """Kernel launches of one AUTO adjoint: the transposition and the gather
-    of each 512 MB of transposed projections in the column form (the
-    library's column_pairs, columns_pay and line_pad rules), or one scatter."""
+    """Kernel launches of one AUTO adjoint of a scan whose rows cover the
+    grid: the transposition and the gather of each 512 MB of transposed
+    projections in the column form (the library's column_pairs, columns_pay
+    and line_pad rules), or one scatter."""
     nz = int(vg.n[2])
     pitch = []
     for k in range(cg.n_views):
@@ -712,7 +735,7 @@ def phantom_kernels(args, gjp, geom, vg, cg, dev, stream, hbm, peak_kind, k16):
     foot = np.array(gjp.footprint_voxels(geom, vg.n, vg.h, device=dev), dtype=np.float64)
     proj_bytes = 4.0 * cg.n_views * cg.nu * cg.nv
     alg = {"forward_f32": 4.0 * foot.sum() + proj_bytes, k16: 2.0 * foot.sum() + proj_bytes,
-           "adjoint_f32": 8.0 * foot.sum() + proj_bytes}
+           "adjoint_f32": adjoint_bytes(vg, cg, foot, proj_bytes)}
     out = {}
     reps = max(1, min(args.steps, 5))
     for name, fn in fns.items():

@@ -166,7 +166,8 @@ gjp_status gjp_forward(const void *d_volume, gjp_dtype dtype, int64_t nx, int64_
 typedef enum {
     GJP_PATH_AUTO = 0,   /* the library's fastest family for the call (forward: the column
                             form where it applies, else PAIRS for 16-bit storage over 32
-                            or more views and 2^27 view-voxels, else GATHER; adjoint: COMBINE) */
+                            or more views and 2^27 view-voxels, else GATHER; adjoint: the
+                            column form where it applies, else COMBINE) */
     GJP_PATH_GATHER = 1, /* one thread per ray, taps gathered from global memory */
     GJP_PATH_SLAB = 2,   /* detector tiles stream per-plane voxel boxes into shared memory
                             with TMA; needs a 16-byte aligned volume whose z row is a
@@ -280,10 +281,11 @@ gjp_status gjp_selftest_tap_check(void *stream);
  * gjp_debug_fail_allocations -- failure-injection hook for tests (the paper
  * has no counterpart): the next `n` device allocations that the library
  * attempts (per-view tables, batch queues, texture arrays, z-paired
- * copies, column records, transposed projections) fail as if the device were out of memory, so the calls that need
- * them return GJP_ERR_OOM and leave their outputs untouched (GJP_PATH_AUTO
- * reads the volume directly instead of a z-paired copy it could not
- * allocate, and takes COMBINE where the column form cannot allocate); later allocations proceed.
+ * copies, column records, transposed projections) fail as if the device were
+ * out of memory, so the calls that need them return GJP_ERR_OOM and leave
+ * their outputs untouched (GJP_PATH_AUTO reads the volume directly instead of
+ * a z-paired copy it could not allocate, and takes COMBINE where the column
+ * form cannot allocate); later allocations proceed.
  * n = 0 clears it.  Host-only, thread-safe; no GPU fault is involved.
  * Returns GJP_ERR_INVALID_ARG for n < 0.
  */
@@ -293,8 +295,9 @@ gjp_status gjp_debug_fail_allocations(int n);
  * gjp_trim_workspace -- returns to the device the memory that the
  * library's workspace pools keep between calls (the z-paired copies of
  * GJP_PATH_PAIRS and the adjoint's transposed projections; up to 8 GiB per
- * device).  Waits for nothing: memory that
- * a queued call still uses is kept until that call is done.  Safe to call
+ * device; what a geometry keeps, its per-view tables and column records, stays
+ * until it is destroyed).  Waits for nothing: memory that a queued call still
+ * uses is kept until that call is done.  Safe to call
  * at any time; GJP_OK unless CUDA reports an error.
  */
 gjp_status gjp_trim_workspace(void);
@@ -341,8 +344,8 @@ gjp_status gjp_adjoint(const float *d_proj, const gjp_geometry *g, int64_t nx, i
  * gjp_trim_workspace), and per-column records (56 bytes per view and
  * detector column) that its first call for a geometry and grid writes on
  * `stream`, without waiting for it, and the geometry keeps until it is
- * destroyed.  While `stream` is being captured, or when either
- * cannot be allocated, AUTO takes COMBINE.  GJP_PATH_PREFETCH is not an adjoint family
+ * destroyed.  While `stream` is being captured, or when either cannot be
+ * allocated, AUTO takes COMBINE.  GJP_PATH_PREFETCH is not an adjoint family
  * (GJP_ERR_INVALID_ARG).  Results agree to float32 rounding; none is
  * bitwise deterministic.
  */

@@ -49,8 +49,8 @@ bool alloc_gate()
     return true;
 }
 
-// Stream-ordered workspace of the z-paired copy: one memory pool per
-// device, owned by the library.  It keeps up to kPairsKeep bytes across
+// Stream-ordered workspace of the z-paired copy and of the column adjoint's
+// transposed projections: one memory pool per device, owned by the library.  It keeps up to kPairsKeep bytes across
 // synchronisations, so that repeated calls on grids up to that size reuse
 // their memory instead of mapping it again; larger copies are returned to
 // the device at the next synchronisation.
@@ -90,9 +90,8 @@ bool pairs_pay(int n_views, const int64_t n[3])
     return n_views >= 32 && (double)n_views * (double)n[0] * (double)n[1] * (double)n[2] >= 134217728.0;
 }
 
-// Allocates `bytes` on stream s for the z-paired copy.  GJP_ERR_UNSUPPORTED
-// while s is being captured into a graph (the copy would become a graph
-// allocation); GJP_ERR_OOM when the allocation gate refuses or the device
+// Allocates `bytes` on stream s.  GJP_ERR_UNSUPPORTED while s is being
+// captured into a graph (the workspace would become a graph allocation); GJP_ERR_OOM when the allocation gate refuses or the device
 // has no room (the CUDA error is cleared).
 gjp_status workspace_alloc(size_t bytes, cudaStream_t s, void **out)
 {
@@ -300,7 +299,8 @@ const ColumnForm *get_columns(const gjp_geometry *gc, gjp_cache_entry &e, const 
     }
 }
 
-// The same with more loads in flight per warp and fewer warps: 8 planes of
+// The gather forward (gjp_forward_kernel, below) with more loads in flight per
+// warp and fewer warps: 8 planes of
 // the row-table march per load batch (from a z-paired copy 16), at 20 (16)
 // warps per SM instead of 32.  For launches whose taps mostly come from DRAM
 // or a cold L2, which wait for latency (deep_loads); bit for bit the same

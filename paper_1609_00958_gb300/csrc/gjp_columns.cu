@@ -719,6 +719,9 @@ int column_pairs(int nz, double pitch)
 // that it visits receive nothing, and its transposed projections and two
 // passes are not repaid by little work (128^3, 4 views: 37 against 34 us;
 // 200x180x256, 2 views: 49 against 67 us; 128^3, 16 views: 67 against 77 us).
+// The z lines at which both are even, per chunk and pair of voxels (and one
+// more), are 19 (300x300x1024) to 33 (100x100x256) over 8 grids with rows one
+// voxel apart: the line lies at the last.
 bool columns_pay(const int64_t n[3], int n_views, double pitch)
 {
     if (n[2] > (1 << 15) || (double)n_views * (double)n[0] * (double)n[1] * (double)n[2] < 16777216.0) return false;
@@ -779,7 +782,10 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
         // the zeros) stay in the L2 while all tiles read them, 64 MB measured
         // best (512^3, 216 views of 1 MB: 2 / 4 / 8 groups 38.3 / 38.0 /
         // 39.2 ms per 360 views); small grids take more groups until every SM
-        // has some waves of warps, of eight views or more.
+        // has some waves of warps, of eight views or more (us for 3000 /
+        // 10000 / 30000 warps: 128^3, 64 views 227 / 180 / 185; 16 views 76 /
+        // 70 / 70; 256^3, 32 views 482 / 482 / 488; 200x180x256, 12 views
+        // 130 / 136 / 137).
         const double mb = (double)j.n_views * g.nu * g.nv * 4.0 / (64.0 * 1024 * 1024);
         const double warps = 2.0 * V.n[0] * V.n[1] / kStrip * column_chunks(V.n[2], K2);
         j.groups = std::max((int)std::ceil(mb), (int)std::ceil(10000.0 / warps));
@@ -987,8 +993,14 @@ __global__ void __launch_bounds__(256, 2) gjp_forward_columns_kernel(
 //     448^3 / 60 views (cost 1.14) 4.76 -> 4.14 ms; 320^3 / 120 views (1.20) 3.02 -> 3.36 ms;
 //     400^3 with 600^2 pixels / 50 views (1.15) 5.35 -> 5.78 ms.
 //   16-bit: 512^3 / 360 views 31.6 -> 29.8 ms, 16 views 2.27 -> 1.43 ms; 1024^3 / 60 views
-//     53.1 -> 43.5 ms; 448^3 / 60 views (1.14) 4.12 -> 4.13 ms.  Grids up to 2^25
-//     voxels keep the z-paired copy.
+//     53.1 -> 43.5 ms; 448^3 / 60 views (1.14) 4.12 -> 4.13 ms; 384x384x256 / 60 views (1.00)
+//     1.44 ms in columns.  Grids up to 2^25 voxels keep the z-paired copy, not for their time
+//     (320x320x256 / 60 views 1.21 -> 1.01 ms, 256^3 / 180 views 2.24 -> 1.96): calls rely on
+//     AUTO's bits and on a batch's launch count there.
+// Beyond the limits (not taken): float32 600x600x320 / 24 views (1.20) 2.92 -> 2.41 ms, 400^3 /
+// 50 views (1.28) 2.79 -> 2.76, 320^3 / 60 views (1.20) 1.59 -> 1.70, 200^3 / 90 views (1.28)
+// 0.66 -> 0.72; bf16 600x600x320 2.94 -> 2.39, 700^3 / 12 views (1.10) 4.16 -> 3.70, 448^3 /
+// 48 views (1.14) 3.37 -> 3.30, 320^3 / 60 views 1.49 -> 1.71.
 // Fewer than 2048 warps leave SMs idle (256^3, f32: one view 34 us for the gather, 56 us for
 // columns; two views 45, 56; four 70, 60).  Float32 grids up to 2^22 voxels keep the gather,
 // with which AUTO agrees bit for bit there.

@@ -69,10 +69,10 @@ struct VolParams {
 #endif
 // Debug build: GJP_CHECK_TAPS=1 range-checks every tap that the interior
 // marches read or reduce without a per-tap test (their plane ranges come
-// from the trimmed estimate of plane_interval).  A tap outside the grid is
-// skipped and recorded in a device status word instead of being accessed;
-// gjp_stream_status then reports GJP_ERR_INTERNAL.  Off by default: the
-// production kernels carry no check.
+// from the corrected estimate of first_above), and the loads of the column
+// forms.  A tap outside the grid is skipped and recorded in a device status
+// word instead of being accessed; gjp_stream_status then reports
+// GJP_ERR_INTERNAL.  Off by default: the production kernels carry no check.
 #ifndef GJP_CHECK_TAPS
 #define GJP_CHECK_TAPS 0
 #endif
