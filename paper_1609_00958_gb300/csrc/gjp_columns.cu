@@ -1,5 +1,6 @@
-// gjp_columns.cu -- the column form of the adjoint: a voxel-driven gather
-// for scans whose detector rows run along z.
+// gjp_columns.cu -- the column forms of the adjoint (a gather driven by the
+// voxels, first below) and of the forward (at the end of the file), for scans
+// whose detector rows run along z.
 //
 // When det_v is parallel to z, all rays of one detector column (fixed view
 // and iu) share their path in (x, y): the same driving axis m, and on plane
@@ -16,16 +17,18 @@
 // memory per voxel, driving axis and view group instead of about two per
 // voxel and view.
 //
-// Measured on 512^3 / 512^2 / 360 views: 38.1 ms, against 68.0 ms for the
-// warp-combined scatter, with a fifth of its error.  Instruction issue bounds
-// it (65% with 16 warps per SM; L1 56%; 24.8 warp instructions per 32 samples of the
-// forward): about 14 instructions for 32 voxels
-// of one column, 30 per column and warp around them, and 1.3 column voxels
-// per sample of the forward (a column at a tile's edge is visited by both
+// Measured on 512^3 / 512^2 / 360 views: 37.2 ms, against 67.7 ms for the
+// warp-combined scatter, with a fifth of its error.  Issue (59%) and the L1
+// (58%) are the busiest units, at the 16 warps per SM that the registers
+// allow; 22.6 warp instructions per 32 samples of the forward, with 1.3
+// column voxels per sample (a column at a tile's edge is visited by both
 // tiles).  8 rows and 256 z fill the registers; fewer rows or a shorter chunk
-// cost more per column (6 rows 44 ms; 128 z 47 ms; 64 z 66 ms), and 4 planes
-// of one strip in a block share the lines in the L1 (90% hits; 8 or 16
-// planes 38.7 and 38.9 ms).
+// cost more per column (of a first version at 38.1 ms: 6 rows 44 ms; 128 z 47
+// ms; 64 z 66 ms), and 4 planes of one strip in a block share the lines in
+// the L1 (90% hits; 8 or 16 planes 38.7 and 38.9 ms).  Ray positions with 23
+// fraction bits in one word took 37.4 ms, but their error grew with the rows'
+// distance (3.6e-7 of the norm on white noise for rows two voxels apart,
+// 1.5e-7 now, 1.8e-7 for the scatter).
 #include "gjp_common.cuh"
 
 namespace gjp_detail {
@@ -780,7 +783,7 @@ gjp_status adjoint_columns(const float *proj, const VolParams &V, const ColumnFo
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         // View groups run one after another: their lines (the values, without
         // the zeros) stay in the L2 while all tiles read them, 64 MB measured
-        // best (512^3, 216 views of 1 MB: 2 / 4 / 8 groups 38.3 / 38.0 /
+        // best (512^3, 216 views of 1 MB, a version at 38.0 ms: 2 / 4 / 8 groups 38.3 / 38.0 /
         // 39.2 ms per 360 views); small grids take more groups until every SM
         // has some waves of warps, of eight views or more (us for 3000 /
         // 10000 / 30000 warps: 128^3, 64 views 227 / 180 / 185; 16 views 76 /
