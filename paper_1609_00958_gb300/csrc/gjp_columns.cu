@@ -133,9 +133,9 @@ bool column_rays(const gjp_geometry &g, const int64_t n[3], const double h[3], c
         const double mid = (g.src[3 * k + 2] - o[2]) / h[2] + t * r0[2], pitch = std::max(std::fabs(t * pv), 1e-9);
         const bool up = t * g.dv[3 * k + 2] > 0.0;
         const double below = (mid + 1.0) / pitch, above = ((double)n[2] - mid) / pitch;   // rows from the middle one
-        const int first = (int)std::max(0.0, std::ceil(cv - (up ? below : above)));
-        const int last = (int)std::min((double)(g.nv - 1), std::floor(cv + (up ? above : below)));
-        inside += std::max(0, last - first + 1) / (double)g.n_views;
+        const double first = std::max(0.0, std::ceil(cv - (up ? below : above)));
+        const double last = std::min((double)(g.nv - 1), std::floor(cv + (up ? above : below)));
+        inside += std::max(0.0, last - first + 1.0) / g.n_views;
         pitch_mean += pitch / g.n_views;
     }
     return rows_pay(c, n, inside, pitch_mean);
@@ -746,7 +746,7 @@ bool columns_pay(const ColumnExtent &x, const int64_t n[3], int n_views)
 {
     if (x.pitch_max > 3.0 || !columns_pay(n, n_views, x.pitch)) return false;
     const double least = x.pitch_mean < 0.53 ? 20.0 : x.pitch_mean < 0.72 ? 42.0 : x.pitch_mean < 1.25 ? 28.0 : 22.0;
-    return x.whole || least * (column_pairs((int)n[2], x.pitch) + 1) * x.chunks <= x.covered;
+    return x.whole || (x.chunks > 0.0 && least * (column_pairs((int)n[2], x.pitch) + 1) * x.chunks <= x.covered);
 }
 
 // Adds A^T proj to vol.

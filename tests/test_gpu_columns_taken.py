@@ -45,3 +45,16 @@ def test_scans_that_do_not(gjp):
     tilted.det_v = tilted.det_v + 1e-3 * tilted.det_u
     assert not _takes(gjp, vg, tilted)
     assert not _takes(gjp, VolumeGeometry.centred((192, 192, 64)), full(12))   # short z lines
+
+
+@pytest.mark.parametrize("offset", [500.0, 1e8, -1e8])
+def test_rows_beyond_the_grid(gjp, offset):
+    """No row meets the grid: nothing is projected back, and no column form is built."""
+    vg = VolumeGeometry.centred((128, 128, 128))
+    cg = synth.circular(12, 130, 140, 500.0, 1000.0, 2.0, angles=0.1 + 0.5 * np.arange(12))
+    cg.src[:, 2] += offset
+    cg.det_origin[:, 2] += offset
+    g = gjp.Geometry.from_cone(cg)
+    y = torch.ones(g.proj_shape, device="cuda")
+    assert float(gjp.adjoint(y, g, vg.n, vg.h).abs().max()) == 0.0
+    assert not takes_columns(gjp, y, g, vg)

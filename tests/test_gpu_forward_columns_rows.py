@@ -43,3 +43,17 @@ def test_rows_beyond_the_grid(gjp, nv, pitch, shift, columns, sign):
     ref = oracle.rays(vol, vg, cg, *rays)
     got = out.cpu().numpy().astype(np.float64)[rays[0], rays[2], rays[1]]
     parity.check_rays(got, vol, vg, cg, *rays, np.abs(ref).max(), TOL32, ref=ref)
+
+
+@pytest.mark.parametrize("offset", [1e8, -1e8])
+def test_rows_far_beyond_the_grid(gjp, offset):
+    """A source and detector 1e8 voxels up or down, rows a fiftieth of a voxel apart: nothing is projected."""
+    vg = VolumeGeometry.centred((190, 180, 128))
+    cg = synth.circular(20, 110, 256, 800.0, 1600.0, 2.3, pitch_v=0.04, angles=0.1 + 0.31 * np.arange(20))
+    cg.src[:, 2] += offset
+    cg.det_origin[:, 2] += offset
+    v = torch.ones(vg.n, device="cuda")
+    g = gjp.Geometry.from_cone(cg)
+    out = gjp.forward(v, g, vg.h)
+    assert torch.equal(out, gjp.forward(v, g, vg.h, path="gather"))
+    assert float(out.abs().max()) == 0.0
